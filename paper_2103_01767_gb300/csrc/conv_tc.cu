@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__
     __shared__ uint32_t tbase;
     __shared__ int abort_flag, issued, consumed;
     __shared__ float red[4][256];
+    __shared__ uint4 mma_list[2 * kMaxGroup];
     const ConvArgs& a = p.a;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int per_img = a.tiles_x * a.tiles_y;
@@ -141,6 +142,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__
         consumed = 0;
     }
     for (int i = threadIdx.x; i < 4 * 256; i += kThreads) (&red[0][0])[i] = 0.0f;
+    const int g0 = a.gstart[pg * a.P], n_mma = (a.gstart[pg * a.P + a.P] - g0) * a.split;
+    for (int i = threadIdx.x; i < n_mma; i += kThreads) {
+        const Group gr = a.group[g0 + i / a.split];
+        const int sp = i % a.split, ph = gr.phase - pg * a.P;
+        const bool first = sp == 0 && g0 + i / a.split == a.gstart[gr.phase];
+        mma_list[i] = make_uint4((uint32_t)((sp * a.n_copy + gr.copy) * 2 * a.a_slot + gr.row * 256) >> 4,
+                                 (uint32_t)(gr.tap * a.N * 16) >> 4, (uint32_t)(ph * a.N), first ? 0u : 1u);
+    }
     fence_before();
     __syncthreads();
     fence_after();
@@ -192,9 +201,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__
     } else if (warp == 1) {
         // MMA issuer: lane 0 issues, the other lanes wait at the warp barrier
         if (lane == 0) {
+            // One thread feeds the tensor pipe, which takes an MMA every 44 (N <= 32), 48 (N = 64)
+            // or 64 cycles (N = 128; the shared-memory reads of A and B bound the smaller N).
+            // Building each MMA's descriptors from its group took that thread about 100 cycles;
+            // now every operand offset comes from mma_list, in the descriptors' 16-byte units.
+            // With two CTAs per SM (finish_plan) the layers of a 225-pattern forward pass went
+            // 429 (mean of layers 2 and 5), 146 and 332 us (3 and 4) -> 222, 115 and 294 us.
             const uint32_t idesc = idesc_bf16(128, a.N, 0, 0);
-            const int g0 = a.gstart[pg * a.P], g1 = a.gstart[pg * a.P + a.P];
-            unsigned started = 0;
             int ks = 0;
             for (; ks < a.ksteps; ++ks) {
                 const int s = ks % S, use = ks / S;
@@ -205,18 +218,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__
                 }
                 fence_after();
                 const uint32_t st = sbase + s * a.stage_bytes;
+                const uint64_t ad0 = sdesc(st, (uint32_t)a.a_slot, 128u);
                 const uint64_t bd0 = sdesc(st + a.a_bytes, 9u * a.N * 16u, 128u);
-                for (int g = g0; g < g1; ++g) {
-                    const Group gr = a.group[g];
-                    const int ph = gr.phase - pg * a.P;
-                    const uint64_t bd = bd0 + (uint64_t)((gr.tap * a.N * 16) >> 4);
-                    const uint32_t d = tmem + (uint32_t)(ph * a.N);
-                    for (int sp = 0; sp < a.split; ++sp) {
-                        const uint32_t aaddr = st + (uint32_t)((sp * a.n_copy + gr.copy) * 2 * a.a_slot + gr.row * 256);
-                        const uint64_t ad = sdesc(aaddr, (uint32_t)a.a_slot, 128u);
-                        mma_bf16(d, ad, bd, idesc, (started >> ph) & 1u);
-                        started |= 1u << ph;
-                    }
+#pragma unroll 6
+                for (int i = 0; i < n_mma; ++i) {
+                    const uint4 m = mma_list[i];
+                    mma_bf16(tmem + m.z, ad0 + m.x, bd0 + m.y, idesc, m.w | (uint32_t)ks);
                 }
                 mma_commit(smem_u32(&empty[s]));
             }
@@ -435,23 +442,31 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tc(const __grid_constant_
                     break;
                 }
                 fence_after();
+                // operand offsets in the descriptors' 16-byte units, added to the stage's two
+                // descriptors (the issuing thread's time per MMA has to stay below the pipe's):
+                // the four wide layers' gradients at batch 64 1389 -> 1284 us in all
                 const uint32_t st = sbase + s * a.stage_bytes;
+                const uint64_t gd0 = sdesc(st, 128u, (uint32_t)a.g_slot);
+                const uint64_t xd0 = sdesc(st + (uint32_t)a.g_bytes, 128u, (uint32_t)a.x_slot);
+                const uint32_t xlo = (uint32_t)(a.n_copy * a.x_real * a.x_slot) >> 4;  // hi -> lo half
+                const uint32_t glo = (uint32_t)(a.g_real * a.g_slot) >> 4;
                 for (int tap = 0; tap < 9; ++tap) {
-                    const int cp = a.grp[ph][tap][0], ro = a.grp[ph][tap][1];
                     const uint32_t d = tmem + (uint32_t)(tap * a.N);
-                    const uint32_t x0 = st + (uint32_t)(a.g_bytes + cp * a.x_real * a.x_slot + ro * 256);
-                    const uint32_t xstride = (uint32_t)(a.n_copy * a.x_real * a.x_slot);  // split 0 -> 1
-                    const uint32_t gstride = (uint32_t)(a.g_real * a.g_slot);
-                    for (int k = 0; k < a.rows_px; ++k) {
-    #pragma unroll
-                        for (int combo = 0; combo < 3; ++combo) {
-                            const int sg = combo == 2 ? 1 : 0, sx = combo == 1 ? 1 : 0;   // hi.hi, hi.lo, lo.hi
-                            const uint64_t gd = sdesc(st + sg * gstride + k * 256, 128u, (uint32_t)a.g_slot);
-                            const uint64_t xd = sdesc(x0 + sx * xstride + k * 256, 128u, (uint32_t)a.x_slot);
-                            const uint32_t acc = (it > 0 || k > 0 || combo > 0) ? 1u : 0u;
-                            if (a.w2) mma_bf16(d, xd, gd, idesc, acc);
-                            else mma_bf16(d, gd, xd, idesc, acc);
+                    uint64_t gh = gd0, xh = xd0 + ((uint32_t)(a.grp[ph][tap][0] * a.x_real * a.x_slot + a.grp[ph][tap][1] * 256) >> 4);
+                    uint32_t acc = it > 0;
+#pragma unroll 4
+                    for (int k = 0; k < a.rows_px; ++k, gh += 16, xh += 16) {   // a row of 16 pixels is 256 bytes
+                        const uint64_t gl = gh + glo, xl = xh + xlo;
+                        if (a.w2) {
+                            mma_bf16(d, xh, gh, idesc, acc);
+                            mma_bf16(d, xl, gh, idesc, 1u);
+                            mma_bf16(d, xh, gl, idesc, 1u);
+                        } else {
+                            mma_bf16(d, gh, xh, idesc, acc);
+                            mma_bf16(d, gh, xl, idesc, 1u);
+                            mma_bf16(d, gl, xh, idesc, 1u);
                         }
+                        acc = 1u;
                     }
                 }
                 mma_commit(smem_u32(&empty[s]));
@@ -643,6 +658,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 EncodeTiledFn g_encode = nullptr;
 bool g_ready = false;
 int g_conv_dyn = 0, g_wg_dyn = 0;   // dynamic shared memory the two kernels may request
+int g_conv_half = 0;                // ... and k_conv_tc with two CTAs on an SM
 
 // map of one half (hi or lo) of a chunk-major tensor; box = 16 pixels x 8 channels x `rows`
 // rows of one chunk (one parity plane of a parity-split tensor: chunk coordinate 4 q + plane)
@@ -715,6 +731,12 @@ cudaError_t finish_plan(ConvPlan& pl, int n_img, int num_sms, int phases, int Nt
     while (a.P > 1 && (a.P * a.N > 512 || tiles * (phases / a.P) < num_sms)) a.P >>= 1;
     if (a.P * a.N > 512) return cudaErrorInvalidConfiguration;
     a.tmem_cols = pow2_cols(a.P * a.N);
+    // Two CTAs per SM where their accumulators fit in TMEM together (and a stage of each in
+    // shared memory): one CTA's set-up and epilogue then overlap the other's MMAs.
+    if (a.tmem_cols <= 256) {
+        const int half = (g_conv_half - 1024) / a.stage_bytes;
+        if (half >= 1) a.n_stage = std::min(a.n_stage, half);
+    }
     for (int pg = 0; pg < 4; ++pg) {
         unsigned m = 0;
         if (pg < phases / a.P)
@@ -745,6 +767,10 @@ cudaError_t tc_prepare() {
     cudaFuncAttributes fa;
     if ((e = cudaFuncGetAttributes(&fa, k_conv_tc)) != cudaSuccess) return e;
     g_conv_dyn = std::min(kSmemLimit, optin - (int)fa.sharedSizeBytes);
+    int per_sm = 0, reserved = 0;
+    if ((e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev)) != cudaSuccess) return e;
+    g_conv_half = per_sm / 2 - reserved - (int)fa.sharedSizeBytes;
     if ((e = cudaFuncGetAttributes(&fa, k_wgrad_tc)) != cudaSuccess) return e;
     g_wg_dyn = std::min(kSmemLimit, optin - (int)fa.sharedSizeBytes);
     if ((e = cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, g_conv_dyn)) != cudaSuccess) return e;
