@@ -374,10 +374,12 @@ __device__ __forceinline__ void gather_joint(float2* v, const float2* __restrict
 }
 
 // Probe block of the adjoint: part[y][x] += conj(C[r0+y][c0+x]) * v[a] in the team's own
-// accumulator row (each element has one owner thread within the team: no atomics).
+// accumulator row (each element has one owner thread within the team: no atomics).  The
+// team's first position stores instead of adding, so nobody has to zero the accumulators
+// (10 MB for 304 teams of 64 x 64 patches).
 template <class G>
 __device__ __forceinline__ void accumulate_probe_adjoint(const float2* v, float2* part, const float2* __restrict__ C,
-                                                         int nx, int r0, int c0, int tid) {
+                                                         int nx, int r0, int c0, int tid, bool first) {
     const int x = tid & (G::S - 1), b = tid >> G::LOG_S;
     const size_t off = (size_t)(r0 + b) * nx + c0 + x;
     const int poff = b * G::S + x;
@@ -391,7 +393,7 @@ __device__ __forceinline__ void accumulate_probe_adjoint(const float2* v, float2
             float2* dst = part + poff + G::BX * G::S * a;
             const float2 t = cconjmul(o, v[a]);
             const float2 cur = *dst;
-            *dst = make_float2(cur.x + t.x, cur.y + t.y);
+            *dst = make_float2((first ? 0.0f : cur.x) + t.x, (first ? 0.0f : cur.y) + t.y);
         }
         sched_fence();
     }
