@@ -24,20 +24,24 @@
 // The last CTA to leave resets the counters (arrivals cnt[0], exits cnt[1], released round
 // cnt[kCoopRelease]) for the next launch.
 #pragma once
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include "griddep.cuh"
 #include "reduce.cuh"
 
 namespace ptylm {
 
-__device__ __forceinline__ float rdotf(float2 a, float2 b) { return a.x * b.x + a.y * b.y; }
+// The CG arithmetic's roundings are written out (fmaf, __fmul_rn), so that its forms, compiled
+// separately, cannot differ in what the compiler contracts.
+__device__ __forceinline__ float rdotf(float2 a, float2 b) { return fmaf(a.x, b.x, __fmul_rn(a.y, b.y)); }
 
 // Jacobi preconditioner z = r / Dg(G + lambda D) = r / ((1 + lambda) D), D = Dg(G)
 // (Sec. 3.3); the identity when D is NULL.
 __device__ __forceinline__ float2 precondition(float2 r, const float* D, float lambda, long i) {
     if (!D) return r;
     const float inv = 1.0f / ((1.0f + lambda) * D[i]);
-    return make_float2(r.x * inv, r.y * inv);
+    return make_float2(__fmul_rn(r.x, inv), __fmul_rn(r.y, inv));
 }
 
 constexpr unsigned kCoopSpinLimit = 1u << 24;   // x >= 32 ns sleep: about a second (the default limit)
@@ -205,6 +209,127 @@ __global__ void __launch_bounds__(256) k_cg_iteration(float2* __restrict__ x, fl
         cnt[1] = 0u;
         __threadfence();
     }
+}
+
+// ---------------------------------------------------------------------------------------
+// The same iteration for short vectors on ONE cluster of 16 CTAs: the two FP64 sums go
+// through distributed shared memory and the cluster's hardware barrier instead of global
+// partials, an arrival counter and polling (5-7 us a round), and x, r, p and q are read once
+// and stay in registers.  Thread t of the 8192 owns the elements t + 8192 j, j < U; the sums
+// are those of the three-launch form on 16 CTAs of 512 threads (per-CTA block sums, then the
+// CTAs in rank order by warp_sum), bit for bit.  It applies where U <= kClusterMaxU, i.e. up
+// to 98,304 elements (313^2); from there on 16 SMs cannot stream the vectors as fast as the
+// whole GPU does.  CTAs of a cluster are scheduled together, so the barrier needs no limit.
+// ---------------------------------------------------------------------------------------
+constexpr int kClusterCtas = 16, kClusterThreads = 512, kClusterMaxU = 12;
+constexpr long kClusterStride = (long)kClusterCtas * kClusterThreads;
+
+// FP64 sum of W per-thread values over the cluster; every thread receives it.  `part` is this
+// call's own [W][kClusterCtas] array.
+template <int W>
+__device__ __forceinline__ void cluster_sum(double (&s)[W], double (*part)[kClusterCtas]) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    block_sum<W>(s);
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int c = 0; c < W; ++c) {
+            const double v = __shfl_sync(0xffffffffu, s[c], 0);
+            if (lane < kClusterCtas) *cl.map_shared_rank(&part[c][cl.block_rank()], lane) = v;
+        }
+    }
+    cl.sync();
+#pragma unroll
+    for (int c = 0; c < W; ++c) s[c] = lane < kClusterCtas ? part[c][lane] : 0.0;
+    warp_sum<W>(s);
+#pragma unroll
+    for (int c = 0; c < W; ++c) s[c] = __shfl_sync(0xffffffffu, s[c], 0);
+}
+
+template <int U>
+__global__ void __launch_bounds__(kClusterThreads) k_cg_cluster(float2* __restrict__ x, float2* __restrict__ r,
+                                                                float2* __restrict__ p, float2* __restrict__ q,
+                                                                const float* __restrict__ D, float lambda, int n,
+                                                                double* sc, double tol) {
+    __shared__ double part1[1][kClusterCtas], part2[2][kClusterCtas];
+    griddep_launch();
+    griddep_wait();   // p . q needs the product launched just before
+    if (tol >= 0.0 && __ldcg(sc + S_CG_DONE) != 0.0) return;  // converged earlier: every CTA sees the same flag
+    const double rz = __ldcg(sc + S_RZ);
+    constexpr int stride = (int)kClusterStride;
+    const int i0 = blockIdx.x * kClusterThreads + threadIdx.x;
+    float2 pv[U], qv[U], xv[U], rv[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+        const int i = i0 + k * stride;
+        pv[k] = qv[k] = xv[k] = rv[k] = make_float2(0.0f, 0.0f);
+        if (i < n) {
+            pv[k] = p[i];
+            qv[k] = q[i];
+            xv[k] = x[i];
+            rv[k] = r[i];
+        }
+    }
+    float f = 0.0f;
+#pragma unroll
+    for (int k = 0; k < U; ++k)
+        if (i0 + k * stride < n) f += rdotf(pv[k], qv[k]);
+    double s1[1] = {f};
+    cluster_sum<1>(s1, part1);
+    const double alpha64 = rz / s1[0];
+    const float alpha = (float)alpha64;
+    float f0 = 0.0f, f1 = 0.0f;
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+        const int i = i0 + k * stride;
+        if (i < n) {
+            xv[k].x += alpha * pv[k].x;
+            xv[k].y += alpha * pv[k].y;
+            rv[k].x -= alpha * qv[k].x;
+            rv[k].y -= alpha * qv[k].y;
+            x[i] = xv[k];
+            r[i] = rv[k];
+            f0 += rdotf(rv[k], precondition(rv[k], D, lambda, i));
+            f1 += rdotf(rv[k], rv[k]);
+        }
+    }
+    double s2[2] = {f0, f1};
+    cluster_sum<2>(s2, part2);
+    const double beta64 = s2[0] / rz;
+    const float beta = (float)beta64;
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+        const int i = i0 + k * stride;
+        if (i < n) {
+            const float2 zi = precondition(rv[k], D, lambda, i);
+            const float2 pn = make_float2(zi.x + beta * pv[k].x, zi.y + beta * pv[k].y);
+            p[i] = pn;
+            const float d = lambda * (D ? D[i] : 1.0f);
+            q[i] = make_float2(d * pn.x, d * pn.y);
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {   // every CTA read S_RZ before the first barrier
+        sc[S_PAP] = s1[0];
+        sc[S_ALPHA] = alpha64;
+        sc[S_RRNEW] = s2[1];
+        sc[S_BETA] = beta64;
+        sc[S_RZ] = s2[0];
+        sc[S_RR] = s2[1];
+        if (tol >= 0.0) {
+            sc[S_CG_ITERS] += 1.0;
+            sc[S_CG_DONE] = sqrt(s2[1]) <= tol ? 1.0 : 0.0;
+        }
+    }
+}
+
+// The kernel for vectors of n elements (NULL: too long for a cluster) and its launch.
+inline const void* cg_cluster_kernel(long n) {
+    const long u = (n + kClusterStride - 1) / kClusterStride;
+    return u > kClusterMaxU ? nullptr
+         : u <= 1 ? (const void*)k_cg_cluster<1> : u <= 2 ? (const void*)k_cg_cluster<2>
+         : u <= 4 ? (const void*)k_cg_cluster<4> : u <= 6 ? (const void*)k_cg_cluster<6>
+         : u <= 9 ? (const void*)k_cg_cluster<9> : (const void*)k_cg_cluster<kClusterMaxU>;
 }
 
 }  // namespace ptylm

@@ -29,7 +29,7 @@ struct PtyArgs {
     const float2* Olin;    // joint: object at the linearisation point (matvec)
     float2* outP_part;     // joint: per-team probe accumulators [grid * TEAMS][M]
     float* trp;            // optional: per-thread sums of d2l [K][T] (forward + cache)
-    const double* skip;    // matvec: return at once when *skip != 0 (a CG solve that has converged)
+    const double* skip;    // matvec in a CG iteration: return at once when *skip != 0 (the solve has converged)
 };
 
 enum KernelId {
@@ -78,7 +78,13 @@ struct CtxView {
 };
 bool ctx_view(const struct ptylm_ctx* c, CtxView* v);
 
-// Launch kernel `kid` for the tile (2^LS side, 2^LE values per thread) on `grid` CTAs.
-cudaError_t kernel_launch(int LS, int LE, int kid, const PtyArgs& a, int grid, cudaStream_t stream);
+// Launch kernel `kid` for the tile (2^LS side, 2^LE values per thread) on `grid` CTAs.  With
+// `dependent` it may start before the kernel launched just before it on the stream has
+// completed (griddep.cuh).  The GGN product then waits for that kernel before its first
+// access when args.skip is set (a CG iteration: the direction comes from that kernel),
+// otherwise before its first accumulation into args.out; the cached forward pass waits before
+// its first accumulation into args.out.  Other kernels must not be launched so.
+cudaError_t kernel_launch(int LS, int LE, int kid, const PtyArgs& a, int grid, cudaStream_t stream,
+                          bool dependent = false);
 
 }  // namespace ptylm

@@ -16,6 +16,7 @@
 //   KID_JVP        J v                                       (App. B Eq. jac_ampl, forward mode)
 #include <type_traits>
 
+#include "griddep.cuh"
 #include "kernels.h"
 #include "ptycho_device.cuh"
 #include "reduce.cuh"
@@ -147,6 +148,7 @@ k_forward(FwdArgs a) {
             if (a.loss == 0) ls.finish<0>(G::E, sl, sd, s2);
             else ls.finish<1>(G::E, sl, sd, s2);
             if (a.trp) a.trp[(size_t)k * G::T + c.tid] = s2;
+            if (k < stride) griddep_wait();   // a.out is zeroed by the kernel before
             if constexpr (FUSED) {
                 const int kn = k + stride;
                 if (kn < a.K) {
@@ -216,7 +218,11 @@ template <int LS, int LE, bool JOINT = false>
 __global__ void __launch_bounds__(Geo<LS, LE>::THREADS, 512 / Geo<LS, LE>::THREADS)
 k_ggn_matvec(MatvecArgs a) {
     using G = Geo<LS, LE>;
-    if (a.skip && __ldcg(a.skip) != 0.0) return;  // every CTA reads the same value
+    griddep_launch();
+    if (a.skip) {
+        griddep_wait();
+        if (__ldcg(a.skip) != 0.0) return;  // every CTA reads the same value
+    }
     TeamCtx<G> c = team_setup<G>(a.tw);
     const float invM = 1.0f / G::M;
     const int stride = gridDim.x * G::TEAMS;
@@ -249,6 +255,7 @@ k_ggn_matvec(MatvecArgs a) {
                 g[k2y] = av[k2y] * t;
             }
         });
+        if (k < stride) griddep_wait();   // a.out holds the damping term from the kernel before
         if constexpr (FUSED) {
             const int kn = k + stride;
             if (kn < a.K) {
@@ -579,7 +586,7 @@ cudaError_t kernel_prepare(int LS, int LE, int kid, int* ctas_per_sm) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, fn, cta_threads(LS, LE), smem);
 }
 
-cudaError_t kernel_launch(int LS, int LE, int kid, const PtyArgs& a, int grid, cudaStream_t stream) {
+cudaError_t kernel_launch(int LS, int LE, int kid, const PtyArgs& a, int grid, cudaStream_t stream, bool dependent) {
     const void* fn = kernel_for(LS, LE, kid);
     if (!fn || grid <= 0) return cudaErrorInvalidValue;
     FwdArgs fa{a.O, a.P, a.pos, a.y, a.a_cache, a.out, a.out_real, a.partials, a.counter, a.scal, a.tw,
@@ -596,7 +603,10 @@ cudaError_t kernel_launch(int LS, int LE, int kid, const PtyArgs& a, int grid, c
         default: arg = &ja; break;
     }
     void* args[] = {arg, &u};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(cta_threads(LS, LE)), args, kernel_smem_bytes(LS, LE, kid), stream);
+    const dim3 block(cta_threads(LS, LE));
+    const size_t smem = kernel_smem_bytes(LS, LE, kid);
+    if (dependent) return launch_dependent(fn, dim3(grid), block, args, smem, stream);
+    return cudaLaunchKernel(fn, dim3(grid), block, args, smem, stream);
 }
 
 }  // namespace ptylm

@@ -17,6 +17,7 @@
 #include "../../include/ptylm.h"
 #include "kernels.h"
 #include "cg_iteration.cuh"
+#include "griddep.cuh"
 #include "reduce.cuh"
 
 using namespace ptylm;
@@ -72,10 +73,23 @@ static constexpr int VEC_THREADS = 256;
 // i of z is vO[i] for i < N, vP[i - N] from there on (joint contexts), and likewise out.
 __global__ void k_damping_init(const float2* __restrict__ vO, const float2* __restrict__ vP, const float* __restrict__ D,
                                float lambda, float2* __restrict__ outO, float2* __restrict__ outP, long N, long n) {
+    griddep_launch();
     GRID_STRIDE(i, n) {
         const float d = lambda * (D ? D[i] : 1.0f);
         const float2 x = i < N ? vO[i] : vP[i - N];
         (i < N ? outO[i] : outP[i - N]) = make_float2(d * x.x, d * x.y);
+    }
+}
+
+// A new linearisation point: O, P into the context's copies and the gradient's L elements
+// zeroed, in one launch (two copies and a memset before).
+__global__ void k_set_point(const float2* __restrict__ O, float2* __restrict__ O_lin, long N, const float2* __restrict__ P,
+                            float2* __restrict__ P_lin, int M, float2* __restrict__ grad, long L) {
+    griddep_launch();
+    GRID_STRIDE(i, L > N + M ? L : N + M) {
+        if (i < N) O_lin[i] = O[i];
+        else if (i < N + M) P_lin[i - N] = P[i - N];
+        if (i < L) grad[i] = make_float2(0.0f, 0.0f);
     }
 }
 
@@ -298,6 +312,8 @@ struct ptylm_ctx {
     int grid[KID_COUNT] = {0};
     int vec_grid = 0;
     int coop_grid = 0;             // grid of the single-launch CG iteration (0: three launches)
+    const void* cluster_cg = nullptr;  // ... or its one-cluster form for short vectors
+    bool polled_cg = false;        // this solve asked for bounded polls: the cooperative form
     int cg_chunk = 1;              // CG iterations the last solve took (the next solve queues as many at once)
     size_t allocated = 0;
     std::vector<void*> allocations;
@@ -410,10 +426,10 @@ static ptylm_status prof_end(ptylm_ctx* c, int id, cudaEvent_t e0, cudaEvent_t e
 }
 
 // Launch a per-position kernel, timing it with events when profiling is on.
-static ptylm_status launch(ptylm_ctx* c, int kid, const PtyArgs& a) {
+static ptylm_status launch(ptylm_ctx* c, int kid, const PtyArgs& a, bool dependent = false) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     STATUS_TRY(prof_begin(c, kid, &e0, &e1));
-    CUDA_TRY(kernel_launch(c->LS, c->LE, kid, a, c->grid[kid], c->stream));
+    CUDA_TRY(kernel_launch(c->LS, c->LE, kid, a, c->grid[kid], c->stream, dependent));
     ++c->launches;
     return prof_end(c, kid, e0, e1);
 }
@@ -524,14 +540,31 @@ static ptylm_status probe_reduce(ptylm_ctx* c, int kid, float2* out, bool accumu
 // Internal operations on device pointers
 // ---------------------------------------------------------------------------------------
 
+static bool aligned8(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 7u) == 0; }
+
+// (O, P) -> (O_lin, P_lin), gradient zeroed; the forward kernel launched next may overlap it.
+static ptylm_status set_point(ptylm_ctx* c, const float2* O, float2* O_lin, const float2* P, float2* P_lin, float2* grad) {
+    k_set_point<<<vec_blocks(c), VEC_THREADS, 0, c->stream>>>(O, O_lin, c->N, P, P_lin, P ? c->M : 0, grad, c->L);
+    return vec_launched(c);
+}
+
 // Forward model + loss; cache=1 also stores a, the linearisation point, the per-thread d2l
 // sums and grad f over z (object part by scatter, probe part by team accumulators).
 static ptylm_status op_forward(ptylm_ctx* c, const float2* O, const float2* P, int cache) {
     const int kid = cache ? (joint(c) ? KID_FWD_CACHE_J : KID_FWD_CACHE) : KID_FWD_LOSS;
+    bool dependent = false;
     if (cache) {
-        if (O != c->O_lin) CUDA_TRY(cudaMemcpyAsync(c->O_lin, O, sizeof(float2) * c->N, cudaMemcpyDeviceToDevice, c->stream));
-        if (P != c->P_lin) CUDA_TRY(cudaMemcpyAsync(c->P_lin, P, sizeof(float2) * c->M, cudaMemcpyDeviceToDevice, c->stream));
-        CUDA_TRY(cudaMemsetAsync(c->grad, 0, sizeof(float2) * c->L, c->stream));
+        // float2 accesses to the caller's point need 8-byte alignment; other pointers are copied first
+        if (O != c->O_lin && P != c->P_lin && aligned8(O) && aligned8(P)) {
+            STATUS_TRY(set_point(c, O, c->O_lin, P, c->P_lin, c->grad));
+            dependent = true;   // the kernel reads (O, P) itself and adds to grad after its FFTs
+        } else {
+            if (O != c->O_lin) CUDA_TRY(cudaMemcpyAsync(c->O_lin, O, sizeof(float2) * c->N, cudaMemcpyDeviceToDevice, c->stream));
+            if (P != c->P_lin) CUDA_TRY(cudaMemcpyAsync(c->P_lin, P, sizeof(float2) * c->M, cudaMemcpyDeviceToDevice, c->stream));
+            CUDA_TRY(cudaMemsetAsync(c->grad, 0, sizeof(float2) * c->L, c->stream));
+            O = c->O_lin;
+            P = c->P_lin;
+        }
         c->has_lin = false;
         c->u_valid = false;
     }
@@ -539,13 +572,13 @@ static ptylm_status op_forward(ptylm_ctx* c, const float2* O, const float2* P, i
         CUDA_TRY(cudaMemsetAsync(c->scal + S_F, 0, 2 * sizeof(double), c->stream));
     } else {
         PtyArgs a = base_args(c);
-        a.O = cache ? c->O_lin : O;
-        a.P = cache ? c->P_lin : P;
+        a.O = O;
+        a.P = P;
         a.a_cache = c->a_cache;
         a.out = c->grad;
         a.counter = c->counters + CNT_FWD;
         a.trp = cache ? c->trp : nullptr;
-        STATUS_TRY(launch(c, kid, a));
+        STATUS_TRY(launch(c, kid, a, dependent));
         if (cache && joint(c)) STATUS_TRY(probe_reduce(c, kid, c->grad + c->N, false));
     }
     if (cache) c->has_lin = c->has_point = true;
@@ -563,7 +596,13 @@ static ptylm_status cg_iteration(ptylm_ctx* c, float2* x, float2* r, float2* p, 
     double* sc = c->scal;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     STATUS_TRY(prof_begin(c, PROF_CG, &e0, &e1));
-    if (!separate && c->coop_grid > 0) {
+    const bool cluster = c->cluster_cg && !c->polled_cg;
+    if (!separate && cluster) {
+        int n32 = (int)n;
+        void* args[] = {&x, &r, &p, &q, &D, &lambda, &n32, &sc, &tol};
+        CUDA_TRY(launch_dependent(c->cluster_cg, dim3(kClusterCtas), dim3(kClusterThreads), args, 0, c->stream, kClusterCtas));
+        ++c->launches;
+    } else if (!separate && c->coop_grid > 0) {
         unsigned* cnt = c->counters + CNT_COOP;
         unsigned spin = c->cg_spin_limit;
         void* args[] = {&x, &r, &p, &q, &D, &lambda, &n, &part, &cnt, &sc, &tol, &spin};
@@ -571,11 +610,14 @@ static ptylm_status cg_iteration(ptylm_ctx* c, float2* x, float2* r, float2* p, 
                                              c->stream));
         ++c->launches;
     } else {
-        STATUS_TRY(dots(c, 1, n, p, q, nullptr, nullptr, nullptr, nullptr, nullptr, S_PAP, OP_ALPHA));
-        const int nb = vec_blocks(c);
-        k_cg_update<<<nb, VEC_THREADS, 0, c->stream>>>(x, r, p, q, D, lambda, n, part, c->counters + CNT_VEC, sc);
+        // the grid of the single-launch form this context uses, so that the sums agree bit for bit
+        const int nb = cluster ? kClusterCtas : vec_blocks(c), nt = cluster ? kClusterThreads : VEC_THREADS;
+        unsigned* cnt = c->counters + CNT_VEC;
+        k_dots<1><<<nb, nt, 0, c->stream>>>(p, q, nullptr, nullptr, nullptr, nullptr, nullptr, n, part, cnt, sc, S_PAP, OP_ALPHA);
+        STATUS_TRY(vec_launched(c));
+        k_cg_update<<<nb, nt, 0, c->stream>>>(x, r, p, q, D, lambda, n, part, cnt, sc);
         STATUS_TRY(vec_launched(c));                                      // x, r; beta
-        k_cg_direction<<<nb, VEC_THREADS, 0, c->stream>>>(r, p, q, D, lambda, n, sc);
+        k_cg_direction<<<nb, nt, 0, c->stream>>>(r, p, q, D, lambda, n, sc);
         STATUS_TRY(vec_launched(c));                                      // p, q = lambda D p
     }
     return prof_end(c, PROF_CG, e0, e1);
@@ -585,16 +627,15 @@ static ptylm_status cg_iteration(ptylm_ctx* c, float2* x, float2* r, float2* p, 
 // the current linearisation) into the look-ahead set; the error metric and ||grad l||^2
 // land in the scalar slots as for any forward pass.
 static ptylm_status op_forward_lookahead(ptylm_ctx* c, const float2* O) {
-    CUDA_TRY(cudaMemcpyAsync(c->O_lin_b, O, sizeof(float2) * c->N, cudaMemcpyDeviceToDevice, c->stream));
-    CUDA_TRY(cudaMemsetAsync(c->grad_b, 0, sizeof(float2) * c->L, c->stream));
+    STATUS_TRY(set_point(c, O, c->O_lin_b, nullptr, nullptr, c->grad_b));
     PtyArgs a = base_args(c);
-    a.O = c->O_lin_b;
+    a.O = O;
     a.P = c->P_lin;
     a.a_cache = c->a_cache_b;
     a.out = c->grad_b;
     a.counter = c->counters + CNT_FWD;
     a.trp = c->trp_b;
-    return launch(c, KID_FWD_CACHE, a);
+    return launch(c, KID_FWD_CACHE, a, true);
 }
 
 // Allocate the look-ahead set once, after everything lm_solve needs; false (and no error)
@@ -649,7 +690,7 @@ static ptylm_status op_matvec_accumulate(ptylm_ctx* c, const float2* vO, const f
         a.VP = vP;
         a.Olin = c->O_lin;
     }
-    STATUS_TRY(launch(c, kid, a));
+    STATUS_TRY(launch(c, kid, a, true));
     if (joint(c)) STATUS_TRY(probe_reduce(c, kid, outP, true));
     return PTYLM_OK;
 }
@@ -828,6 +869,23 @@ ptylm_status lm_init(ptylm_ctx** out, const ptylm_desc* desc, const int32_t* pos
             c->coop_grid = (int)std::min<long>(c->vec_grid, (long)per_sm * c->num_sms);
         cudaGetLastError();
         c->partials_cap = std::max(c->partials_cap, c->coop_grid);   // rounds 1 and 2 use 3 x grid doubles
+        // One cluster for short vectors.  (The three-launch form then runs on as many CTAs, whose
+        // partial sums have to fit.)
+        const void* fn = c->coop_grid > 0 && c->partials_cap >= kClusterCtas ? cg_cluster_kernel(c->L) : nullptr;
+        if (fn && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute at;
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = kClusterCtas;
+            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            cfg.gridDim = dim3(kClusterCtas);
+            cfg.blockDim = dim3(kClusterThreads);
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            int clusters = 0;
+            if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters > 0) c->cluster_cg = fn;
+        }
+        cudaGetLastError();
     }
 
     ptylm_status s;
@@ -1080,7 +1138,9 @@ ptylm_status ggn_matvec(ptylm_ctx* c, const ptylm_c64* vO, const ptylm_c64* vP, 
     };
     const bool aliased = joint(c) && (overlap(v, nb, o, nb) || overlap(v, nb, u, mb) || overlap(w, mb, o, nb) ||
                                       overlap(w, mb, u, mb));
-    const bool stage_in = host_in || aliased, stage_out = host_out;
+    // ... and joint vectors that float2 accesses cannot take
+    const bool stage_in = host_in || aliased || (joint(c) && !(aligned8(v) && aligned8(w)));
+    const bool stage_out = host_out || (joint(c) && !(aligned8(o) && aligned8(u)));
     if (stage_in && !c->stage_a) STATUS_TRY(ctx_alloc_t(c, &c->stage_a, c->L, "staging (vector)"));
     if (stage_out && !c->stage_b) STATUS_TRY(ctx_alloc_t(c, &c->stage_b, c->L, "staging (result)"));
     if (stage_in) {
@@ -1117,6 +1177,7 @@ static ptylm_status lm_solve_impl(ptylm_ctx* c, ptylm_c64* O_inout, ptylm_c64* P
     if (prm->max_outer < 0 || prm->max_cg < 0 || !(prm->kappa > 1.0) || !(prm->mu0 > 0.0) || prm->wait_polls < 0)
         return fail(PTYLM_ERR_ARG, "invalid LM parameters");
     c->cg_spin_limit = prm->wait_polls > 0 ? (unsigned)prm->wait_polls : kCoopSpinLimit;
+    c->polled_cg = prm->wait_polls > 0;
     if (prm->projected && (!(prm->radius_O > 0.0) || !(prm->radius_P > 0.0) || prm->max_ls < 0))
         return fail(PTYLM_ERR_ARG, "invalid projection parameters");
     if (c->d.K == 0) return fail(PTYLM_ERR_ARG, "lm_solve needs at least one scan position");
@@ -1308,7 +1369,7 @@ static ptylm_status lm_solve_impl(ptylm_ctx* c, ptylm_c64* O_inout, ptylm_c64* P
                         if (std::sqrt(c->scal_host[S_RR]) <= tol) { converged = true; break; }
                         if (it >= prm->max_cg) break;
                     }
-                    STATUS_TRY(op_matvec_accumulate(c, p, p + N, q, q + N));              // q += G p
+                    STATUS_TRY(op_matvec_accumulate(c, p, p + N, q, q + N, c->scal + S_ZERO));      // q += G p
                     ++matvecs;
                     STATUS_TRY(cg_iteration(c, x, r, p, q, D, lam32, separate));
                     ++it;

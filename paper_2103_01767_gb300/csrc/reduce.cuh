@@ -22,6 +22,7 @@ enum Slot {
     S_FMIN = 18,                        // Poisson: sum y - y log y
     S_CG_TIMEOUT = 19,                  // set when a wait of the single-launch CG iteration gave up
     S_CG_DONE = 20, S_CG_ITERS = 21,    // device-side CG stopping: converged flag, iterations run
+    S_ZERO = 23,                        // never written after the context's set-up: a skip flag that is not set
     S_COUNT = 24
 };
 
