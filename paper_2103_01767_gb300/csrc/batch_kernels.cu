@@ -38,17 +38,13 @@ __device__ __forceinline__ void batch_fill_twiddles(float2* tw, const float2* w_
     fill_twiddles<Geo<7, 5>>(tw + batch_tw_offset<Geo<7, 5>>(), w_all + 96, threadIdx.x, blockDim.x);
 }
 
-// Sum two per-thread doubles over the warp and add them to f[0], f[1].
-__device__ __forceinline__ void warp_add_to(double* f, double x, double y) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        x += __shfl_xor_sync(0xffffffffu, x, o);
-        y += __shfl_xor_sync(0xffffffffu, y, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(f, x);
-        atomicAdd(f + 1, y);
-    }
+// Sum two per-thread pairs over the warp and add them to the FP64 totals f[0], f[1] (lane 0
+// and lane 1 together: FP64 in one instruction each, see reduce.cuh).
+__device__ __forceinline__ void warp_add_to(double* f, SumPair x, SumPair y) {
+    x = pair_tree<32>(x);
+    y = pair_tree<32>(y);
+    const int lane = threadIdx.x & 31;
+    if (lane < 2) atomicAdd(f + lane, (double)(lane ? y.h : x.h) + (double)(lane ? y.l : x.l));
 }
 
 // Forward model, error metric and (CACHE) cache a and gradient for one item.
@@ -62,7 +58,7 @@ __device__ __forceinline__ void batch_forward_item(const BatchArgs& a, const Bat
     const float invS = 1.0f / G::S;
     const float2* O = a.V + p.z_off;
     float2* gout = a.out + p.z_off;
-    double acc_l = 0.0, acc_d = 0.0;
+    SumPair acc_l = {}, acc_d = {};
     float2 v[G::E];
     for (int j = 0; j < it.per_team; ++j) {
         const int k = it.k0 + team + TEAMS * j;
@@ -114,8 +110,8 @@ __device__ __forceinline__ void batch_forward_item(const BatchArgs& a, const Bat
         if (p.loss == 0) ls.finish<0>(G::E, sl, sd, s2);
         else ls.finish<1>(G::E, sl, sd, s2);
         if (valid) {
-            acc_l += (double)sl;
-            acc_d += (double)sd;
+            pair_add(acc_l, sl);
+            pair_add(acc_d, sd);
             if constexpr (CACHE) p.trp[(size_t)k * G::T + tid] = s2;   // for the closed-form diagonal
         }
         team_sync<G>();
@@ -257,9 +253,10 @@ __global__ void __launch_bounds__(256) k_batch_diag(const BatchProblem* __restri
     const BatchProblem p = probs[b];
     const int k = g - pos_first[b];
     const int S = 1 << p.LS, M = S * S, T = M >> p.LE;
-    double s[1] = {0.0};
-    for (int t = threadIdx.x; t < T; t += blockDim.x) s[0] += (double)p.trp[(size_t)k * T + t];
-    block_sum<1>(s);
+    SumPair v[1] = {};
+    for (int t = threadIdx.x; t < T; t += blockDim.x) pair_add(v[0], p.trp[(size_t)k * T + t]);
+    double s[1];
+    block_sum<1>(v, s);
     __shared__ float scale;
     if (threadIdx.x == 0) scale = (float)s[0] / (2.0f * (float)M);
     __syncthreads();

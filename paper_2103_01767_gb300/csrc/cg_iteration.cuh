@@ -38,10 +38,12 @@ __device__ __forceinline__ float rdotf(float2 a, float2 b) { return fmaf(a.x, b.
 
 // Jacobi preconditioner z = r / Dg(G + lambda D) = r / ((1 + lambda) D), D = Dg(G)
 // (Sec. 3.3); the identity when D is NULL.
-__device__ __forceinline__ float2 precondition(float2 r, const float* D, float lambda, long i) {
-    if (!D) return r;
-    const float inv = 1.0f / ((1.0f + lambda) * D[i]);
+__device__ __forceinline__ float2 precondition(float2 r, float d, float lambda) {
+    const float inv = 1.0f / ((1.0f + lambda) * d);
     return make_float2(__fmul_rn(r.x, inv), __fmul_rn(r.y, inv));
+}
+__device__ __forceinline__ float2 precondition(float2 r, const float* D, float lambda, long i) {
+    return D ? precondition(r, D[i], lambda) : r;
 }
 
 constexpr unsigned kCoopSpinLimit = 1u << 24;   // x >= 32 ns sleep: about a second (the default limit)
@@ -69,10 +71,11 @@ __device__ __forceinline__ unsigned atom_add_acq_rel_gpu(unsigned* p, unsigned v
 // arrival is an acquire-release add (it publishes the CTA's partial and, for the last CTA,
 // makes every partial visible); the release is a release store read by acquire loads.
 template <int W>
-__device__ void coop_reduce_round(double (&s)[W], double* part, unsigned* cnt, double* sc, int op, unsigned round,
+__device__ void coop_reduce_round(const float (&f)[W], double* part, unsigned* cnt, double* sc, int op, unsigned round,
                                   unsigned spin_limit, double tol = -1.0) {
     __shared__ bool is_last;
-    block_sum<W>(s);
+    double s[W];
+    block_sum<W>(f, s);
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int c = 0; c < W; ++c) part[blockIdx.x * W + c] = s[c];
@@ -82,12 +85,7 @@ __device__ void coop_reduce_round(double (&s)[W], double* part, unsigned* cnt, d
     __syncthreads();
     if (is_last) {
         double t[W];
-#pragma unroll
-        for (int c = 0; c < W; ++c) t[c] = 0.0;
-        for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
-#pragma unroll
-            for (int c = 0; c < W; ++c) t[c] += __ldcg(part + b * W + c);
-        block_sum<W>(t);
+        sum_partials<W>(part, W, gridDim.x, t);
         if (threadIdx.x == 0) {
             apply_final_op(t, W, sc, 0, op);
             if (tol >= 0.0) {  // the CG stopping test ||r|| <= tol, taken on the device
@@ -139,7 +137,7 @@ __global__ void __launch_bounds__(256) k_cg_iteration(float2* __restrict__ x, fl
         for (int k = 0; k < U; ++k)
             if (base + k * stride < n) f += rdotf(pv[k], qv[k]);
     }
-    double s1[1] = {f};
+    const float s1[1] = {f};
     coop_reduce_round<1>(s1, part, cnt, sc, OP_ALPHA, 1u, spin_limit);
     const float alpha = (float)__ldcg(sc + S_ALPHA);
 
@@ -174,7 +172,7 @@ __global__ void __launch_bounds__(256) k_cg_iteration(float2* __restrict__ x, fl
             }
         }
     }
-    double s2[2] = {f0, f1};
+    const float s2[2] = {f0, f1};
     coop_reduce_round<2>(s2, part + gridDim.x, cnt, sc, OP_BETA, 2u, spin_limit, tol);
     const float beta = (float)__ldcg(sc + S_BETA);
 
@@ -224,27 +222,26 @@ __global__ void __launch_bounds__(256) k_cg_iteration(float2* __restrict__ x, fl
 constexpr int kClusterCtas = 16, kClusterThreads = 512, kClusterMaxU = 12;
 constexpr long kClusterStride = (long)kClusterCtas * kClusterThreads;
 
-// FP64 sum of W per-thread values over the cluster; every thread receives it.  `part` is this
-// call's own [W][kClusterCtas] array.
+// FP64 sums of W <= 2 per-thread values over the cluster, for warp 0 (all its lanes).
+// `part` is this call's own [W][kClusterCtas] array.
 template <int W>
-__device__ __forceinline__ void cluster_sum(double (&s)[W], double (*part)[kClusterCtas]) {
+__device__ __forceinline__ void cluster_sum(const float (&f)[W], double (&s)[W], double (*part)[kClusterCtas]) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
-    block_sum<W>(s);
+    block_sum<W>(f, s);
     const int lane = threadIdx.x & 31;
-    if (threadIdx.x < 32) {
+    if (threadIdx.x < kClusterCtas) {
 #pragma unroll
-        for (int c = 0; c < W; ++c) {
-            const double v = __shfl_sync(0xffffffffu, s[c], 0);
-            if (lane < kClusterCtas) *cl.map_shared_rank(&part[c][cl.block_rank()], lane) = v;
-        }
+        for (int c = 0; c < W; ++c) *cl.map_shared_rank(&part[c][cl.block_rank()], lane) = s[c];
     }
     cl.sync();
+    if (threadIdx.x < 32) {   // lanes 16 c + r: CTA r's partial of column c
+        double t = lane < W * kClusterCtas ? part[lane / kClusterCtas][lane % kClusterCtas] : 0.0;
 #pragma unroll
-    for (int c = 0; c < W; ++c) s[c] = lane < kClusterCtas ? part[c][lane] : 0.0;
-    warp_sum<W>(s);
+        for (int o = kClusterCtas / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
 #pragma unroll
-    for (int c = 0; c < W; ++c) s[c] = __shfl_sync(0xffffffffu, s[c], 0);
+        for (int c = 0; c < W; ++c) s[c] = __shfl_sync(0xffffffffu, t, c * kClusterCtas);
+    }
 }
 
 template <int U>
@@ -253,6 +250,7 @@ __global__ void __launch_bounds__(kClusterThreads) k_cg_cluster(float2* __restri
                                                                 const float* __restrict__ D, float lambda, int n,
                                                                 double* sc, double tol) {
     __shared__ double part1[1][kClusterCtas], part2[2][kClusterCtas];
+    __shared__ float ratio[2];   // alpha, beta
     griddep_launch();
     griddep_wait();   // p . q needs the product launched just before
     if (tol >= 0.0 && __ldcg(sc + S_CG_DONE) != 0.0) return;  // converged earlier: every CTA sees the same flag
@@ -260,25 +258,33 @@ __global__ void __launch_bounds__(kClusterThreads) k_cg_cluster(float2* __restri
     constexpr int stride = (int)kClusterStride;
     const int i0 = blockIdx.x * kClusterThreads + threadIdx.x;
     float2 pv[U], qv[U], xv[U], rv[U];
+    float dv[U];   // D, so that the loads of all five vectors are in flight together
 #pragma unroll
     for (int k = 0; k < U; ++k) {
         const int i = i0 + k * stride;
         pv[k] = qv[k] = xv[k] = rv[k] = make_float2(0.0f, 0.0f);
+        dv[k] = 1.0f;
         if (i < n) {
             pv[k] = p[i];
             qv[k] = q[i];
             xv[k] = x[i];
             rv[k] = r[i];
+            if (D) dv[k] = D[i];
         }
     }
     float f = 0.0f;
 #pragma unroll
     for (int k = 0; k < U; ++k)
         if (i0 + k * stride < n) f += rdotf(pv[k], qv[k]);
-    double s1[1] = {f};
-    cluster_sum<1>(s1, part1);
-    const double alpha64 = rz / s1[0];
-    const float alpha = (float)alpha64;
+    const float f1v[1] = {f};
+    double s1[1], alpha64 = 0.0, beta64 = 0.0;
+    cluster_sum<1>(f1v, s1, part1);
+    if (threadIdx.x < 32) {
+        alpha64 = rz / s1[0];
+        if (threadIdx.x == 0) ratio[0] = (float)alpha64;
+    }
+    __syncthreads();
+    const float alpha = ratio[0];
     float f0 = 0.0f, f1 = 0.0f;
 #pragma unroll
     for (int k = 0; k < U; ++k) {
@@ -290,22 +296,27 @@ __global__ void __launch_bounds__(kClusterThreads) k_cg_cluster(float2* __restri
             rv[k].y -= alpha * qv[k].y;
             x[i] = xv[k];
             r[i] = rv[k];
-            f0 += rdotf(rv[k], precondition(rv[k], D, lambda, i));
+            f0 += rdotf(rv[k], D ? precondition(rv[k], dv[k], lambda) : rv[k]);
             f1 += rdotf(rv[k], rv[k]);
         }
     }
-    double s2[2] = {f0, f1};
-    cluster_sum<2>(s2, part2);
-    const double beta64 = s2[0] / rz;
-    const float beta = (float)beta64;
+    const float f2v[2] = {f0, f1};
+    double s2[2];
+    cluster_sum<2>(f2v, s2, part2);
+    if (threadIdx.x < 32) {
+        beta64 = s2[0] / rz;
+        if (threadIdx.x == 0) ratio[1] = (float)beta64;
+    }
+    __syncthreads();
+    const float beta = ratio[1];
 #pragma unroll
     for (int k = 0; k < U; ++k) {
         const int i = i0 + k * stride;
         if (i < n) {
-            const float2 zi = precondition(rv[k], D, lambda, i);
+            const float2 zi = D ? precondition(rv[k], dv[k], lambda) : rv[k];
             const float2 pn = make_float2(zi.x + beta * pv[k].x, zi.y + beta * pv[k].y);
             p[i] = pn;
-            const float d = lambda * (D ? D[i] : 1.0f);
+            const float d = lambda * dv[k];
             q[i] = make_float2(d * pn.x, d * pn.y);
         }
     }

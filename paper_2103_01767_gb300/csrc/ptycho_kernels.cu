@@ -87,7 +87,7 @@ k_forward(FwdArgs a) {
     using G = Geo<LS, LE>;
     TeamCtx<G> c = team_setup<G>(a.tw);
     const float invS = 1.0f / G::S;
-    double acc_l = 0.0, acc_d = 0.0;
+    SumPair acc[2] = {};   // l and dl^2 over this thread's pixels of all its positions
     const int ky = freq_ky<G>(c.tid);
     const int stride = gridDim.x * G::TEAMS;
     // 128^2 object-only linearisations fuse each position's gradient scatter with the next
@@ -201,12 +201,11 @@ k_forward(FwdArgs a) {
                 else pixels(std::integral_constant<int, 1>{});
             }
         }
-        acc_l += (double)sl;
-        acc_d += (double)sd;
+        pair_add(acc[0], sl);
+        pair_add(acc[1], sd);
         team_sync<G>();
     }
-    double sums[2] = {acc_l, acc_d};
-    if constexpr (!INTENSITY && !MAG) grid_reduce<2>(sums, a.partials, a.counter, a.scal, S_F, OP_STORE, 1.0);
+    if constexpr (!INTENSITY && !MAG) grid_reduce<2>(acc, a.partials, a.counter, a.scal, S_F, OP_STORE);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -444,8 +443,9 @@ k_diag_object(const float* __restrict__ trp, const int2* __restrict__ pos, const
               float* D_O, float* tr) {
     using G = Geo<LS, LE>;
     const int k = blockIdx.x, tid = threadIdx.x;
-    double s[1] = {(double)trp[(size_t)k * G::T + tid]};
-    block_sum<1>(s);
+    const float v[1] = {trp[(size_t)k * G::T + tid]};
+    double s[1];
+    block_sum<1>(v, s);
     __shared__ float trk;
     if (tid == 0) {
         trk = (float)s[0];
@@ -463,9 +463,10 @@ k_diag_object(const float* __restrict__ trp, const int2* __restrict__ pos, const
     }
 }
 
-// One block per 32 probe pixels: warp w sums the positions k = w (mod 32), the warp sums are
-// added in warp order.  (One thread per pixel over all positions left M / 256 CTAs of serial
-// loads: 44 us at 64^2 / 400 positions, 4.6 us now.)
+// One block per 32 probe pixels.  The 32 warps fetch |O|^2 of 32 positions at a time into
+// shared memory; warp 0 adds them position by position (the order of one thread running over
+// all positions) while the others fetch the next 32.  (With one thread per pixel M / 256 CTAs
+// waited for one load after another: 44.4 us at 64^2 / 400 positions.)
 template <int LS, int LE>
 __global__ void __launch_bounds__(1024) k_diag_probe(const float* __restrict__ tr, const int2* __restrict__ pos, int K,
                                                      const float2* __restrict__ O, int nx, float* D_P) {
@@ -473,22 +474,38 @@ __global__ void __launch_bounds__(1024) k_diag_probe(const float* __restrict__ t
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int m = blockIdx.x * 32 + lane;
     const int y = m >> G::LOG_S, x = m & (G::S - 1);
+    __shared__ float o2[2][32][32], trs[2][32];
+    constexpr int AHEAD = 8;   // fetches each warp has in flight
     float acc = 0.0f;
-#pragma unroll 4
-    for (int k = w; k < K; k += 32) {
-        const int2 rc = pos[k];
-        const float2 o = O[(size_t)(rc.x + y) * nx + rc.y + x];
-        acc += (o.x * o.x + o.y * o.y) * tr[k];
-    }
-    __shared__ float part[32][32];
-    part[w][lane] = acc;
-    __syncthreads();
-    if (w == 0) {
-        float s = 0.0f;
+    int buf = 0;
+    for (int k0 = 0; k0 < K; k0 += 32 * AHEAD) {
+        float v[AHEAD], t[AHEAD];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) s += part[i][lane];
-        D_P[m] = s / (2.0f * G::M);
+        for (int j = 0; j < AHEAD; ++j) {
+            const int k = k0 + 32 * j + w;
+            v[j] = t[j] = 0.0f;
+            if (k < K) {
+                const int2 rc = pos[k];
+                const float2 o = O[(size_t)(rc.x + y) * nx + rc.y + x];
+                v[j] = o.x * o.x + o.y * o.y;
+                t[j] = tr[k];
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < AHEAD; ++j) {
+            const int n = min(32, K - k0 - 32 * j);
+            if (n <= 0) break;
+            o2[buf][w][lane] = v[j];
+            if (lane == 0) trs[buf][w] = t[j];
+            __syncthreads();   // buffer `buf` is full, and buffer buf ^ 1 has been added up
+            if (w == 0) {
+#pragma unroll 8
+                for (int i = 0; i < n; ++i) acc = fmaf(o2[buf][i][lane], trs[buf][i], acc);
+            }
+            buf ^= 1;
+        }
     }
+    if (w == 0) D_P[m] = acc / (2.0f * G::M);
 }
 
 cudaError_t launch_ggn_diag(int LS, int LE, const float* trp, const int2* pos, int K, const float2* O, const float2* P,

@@ -108,10 +108,7 @@ __global__ void k_dots(const float2* __restrict__ a0, const float2* __restrict__
         if constexpr (W > 1) f[1] += rdotf(a1[i], b1[i]);
         if constexpr (W > 2) f[2] += rdotf(a2[i], b2[i]);
     }
-    double s[W];
-#pragma unroll
-    for (int c = 0; c < W; ++c) s[c] = f[c];
-    grid_reduce<W>(s, part, counter, sc, dst, op, 1.0);
+    grid_reduce<W>(f, part, counter, sc, dst, op);
 }
 
 // CG start: r = -g - q, z = precond(r), p = z, q = lambda D p; r.z and r.r into the slots.
@@ -130,8 +127,8 @@ __global__ void k_cg_start(const float2* __restrict__ g, float2* __restrict__ q,
         f0 += rdotf(ri, zi);
         f1 += rdotf(ri, ri);
     }
-    double s[2] = {f0, f1};
-    grid_reduce<2>(s, part, counter, sc, 0, OP_START, 1.0);
+    const float s[2] = {f0, f1};
+    grid_reduce<2>(s, part, counter, sc, 0, OP_START);
 }
 
 // The stopping test before the first CG iteration, taken on the device: S_CG_DONE =
@@ -161,8 +158,8 @@ __global__ void k_cg_update(float2* __restrict__ x, float2* __restrict__ r, cons
         f0 += rdotf(ri, precondition(ri, D, lambda, i));
         f1 += rdotf(ri, ri);
     }
-    double s[2] = {f0, f1};
-    grid_reduce<2>(s, part, counter, sc, 0, OP_BETA, 1.0);
+    const float s[2] = {f0, f1};
+    grid_reduce<2>(s, part, counter, sc, 0, OP_BETA);
 }
 
 // p = precond(r) + beta p;  q = lambda D p (starts the next matvec's accumulator).
@@ -208,37 +205,48 @@ __global__ void k_poisson_fmin(const float* __restrict__ y, long n, double* part
         const float v = y[i];
         f += v - (v > 0.0f ? v * logf(v) : 0.0f);
     }
-    double s[1] = {f};
-    grid_reduce<1>(s, part, counter, sc, S_FMIN, OP_STORE, 1.0);
+    const float s[1] = {f};
+    grid_reduce<1>(s, part, counter, sc, S_FMIN, OP_STORE);
 }
 
-// Probe block of an adjoint: out[m] (+)= sum over team slots of part[slot][m].  A block sums
-// 32 probe pixels (256 contiguous bytes of a slot): warp w the slots w, w + 32, ... in order,
-// then the warp sums in warp order, the same order every time.  (One thread per pixel over
-// all slots left M / 256 CTAs of serial loads: 34.9 us for 304 slots of 64 x 64, 3.6 us now.)
+// Probe block of an adjoint: out[m] (+)= sum over team slots of part[slot][m], slots in order.
+// A block sums 32 probe pixels (256 contiguous bytes of a slot): its 32 warps fetch 32 slots at
+// a time into shared memory, warp 0 adds them in slot order while the others fetch the next
+// 32.  (One thread per pixel left M / 256 CTAs waiting for one load after another: 34.9 us for
+// 304 slots of 64 x 64.)
 __global__ void __launch_bounds__(1024) k_probe_reduce(const float2* __restrict__ part, int slots, int M,
                                                        float2* __restrict__ out, int accumulate) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int m = blockIdx.x * 32 + lane;   // M is a multiple of 32
+    __shared__ float2 val[2][32][32];
+    constexpr int AHEAD = 8;   // fetches each warp has in flight
     float2 acc = make_float2(0.0f, 0.0f);
-#pragma unroll 8
-    for (int s = w; s < slots; s += 32) {
-        const float2 v = part[(size_t)s * M + m];
-        acc.x += v.x;
-        acc.y += v.y;
-    }
-    __shared__ float2 sums[32][32];
-    sums[w][lane] = acc;
-    __syncthreads();
-    if (w == 0) {
-        float2 t = accumulate ? out[m] : make_float2(0.0f, 0.0f);
+    if (w == 0 && accumulate) acc = out[m];
+    int buf = 0;
+    for (int s0 = 0; s0 < slots; s0 += 32 * AHEAD) {
+        float2 v[AHEAD];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            t.x += sums[i][lane].x;
-            t.y += sums[i][lane].y;
+        for (int j = 0; j < AHEAD; ++j) {
+            const int s = s0 + 32 * j + w;
+            v[j] = s < slots ? part[(size_t)s * M + m] : make_float2(0.0f, 0.0f);
         }
-        out[m] = t;
+#pragma unroll
+        for (int j = 0; j < AHEAD; ++j) {
+            const int n = min(32, slots - s0 - 32 * j);
+            if (n <= 0) break;
+            val[buf][w][lane] = v[j];
+            __syncthreads();   // buffer `buf` is full, and buffer buf ^ 1 has been added up
+            if (w == 0) {
+#pragma unroll 8
+                for (int i = 0; i < n; ++i) {
+                    acc.x += val[buf][i][lane].x;
+                    acc.y += val[buf][i][lane].y;
+                }
+            }
+            buf ^= 1;
+        }
     }
+    if (w == 0) out[m] = acc;
 }
 
 // The diagonal floor acts on two blocks with their own maxima, the object [0, N) and the
@@ -290,8 +298,7 @@ __global__ void k_err_sums(const float2* __restrict__ O, const float2* __restric
         f[2] += o.x * o.x + o.y * o.y;
         f[3] += r.x * r.x + r.y * r.y;
     }
-    double s[4] = {f[0], f[1], f[2], f[3]};
-    grid_reduce<4>(s, part, counter, sc, S_ER, OP_STORE, 1.0);
+    grid_reduce<4>(f, part, counter, sc, S_ER, OP_STORE);
 }
 
 // ---------------------------------------------------------------------------------------

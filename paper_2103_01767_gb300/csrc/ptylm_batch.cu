@@ -149,10 +149,11 @@ struct DotArgs {
 
 // Per chunk partial sums -> per problem FP64 sums (chunk order) -> op and CG bookkeeping.
 template <int W>
-__device__ void batch_finish(const DotArgs& d, double (&s)[W]) {
+__device__ void batch_finish(const DotArgs& d, const float (&f)[W]) {
     __shared__ bool is_last;
     __shared__ int s_any;
-    block_sum<W>(s);
+    double s[W];
+    block_sum<W>(f, s);
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int w = 0; w < W; ++w) d.part[blockIdx.x * 4 + w] = s[w];
@@ -163,19 +164,31 @@ __device__ void batch_finish(const DotArgs& d, double (&s)[W]) {
     __syncthreads();
     if (!is_last) return;
     __threadfence();
-    for (int b = threadIdx.x; b < d.B; b += blockDim.x) {
-        const bool in = d.post == POST_START ? (d.lm_active == nullptr || d.lm_active[b] != 0)
-                                             : (d.mask == nullptr || d.mask[b] != 0);
+    // eight lanes per problem and column load the chunk partials together and add them; a warp
+    // takes 32 / (8 columns) problems at a time, so that each FP64 instruction (64 cycles,
+    // reduce.cuh) serves all of its lanes.  (One thread per problem went through up to 64
+    // partials one after another.)
+    constexpr int COLS = W == 1 ? 1 : W == 2 ? 2 : 4, PROBS = 4 / COLS;
+    const int lane = threadIdx.x & 31, col = (lane >> 3) % COLS, grp = lane / (8 * COLS);
+    for (int b0 = (threadIdx.x >> 5) * PROBS; b0 < d.B; b0 += (blockDim.x >> 5) * PROBS) {
+        const int b = b0 + grp;
+        const bool in = b < d.B && (d.post == POST_START ? (d.lm_active == nullptr || d.lm_active[b] != 0)
+                                                         : (d.mask == nullptr || d.mask[b] != 0));
+        double v = 0.0;
+        if (in && col < W) {
+            const int q1 = d.chunk_first[b + 1];
+            for (int q = d.chunk_first[b] + (lane & 7); q < q1; q += 8) v += __ldcg(d.part + (size_t)q * 4 + col);
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        double t[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) t[w] = __shfl_sync(0xffffffffu, v, 8 * (COLS * grp + w));
+        if (lane % (8 * COLS) != 0 || b >= d.B) continue;
         if (!in) {
             if (d.post == POST_START) d.mask[b] = 0;   // problems not solving take no CG iteration
             continue;
         }
-        double t[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) t[w] = 0.0;
-        for (int q = d.chunk_first[b]; q < d.chunk_first[b + 1]; ++q)
-#pragma unroll
-            for (int w = 0; w < W; ++w) t[w] += __ldcg(d.part + q * 4 + w);
         double* sc = d.sc + (size_t)b * S_COUNT;
         apply_final_op(t, W, sc, d.dst, d.op);
         if (d.post == POST_START) {
@@ -215,10 +228,7 @@ __global__ void kb_dots(DotArgs d, const float2* __restrict__ a0, const float2* 
             if constexpr (W > 2) f[2] += brdot(a2[g], b2[g]);
         }
     }
-    double s[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) s[w] = f[w];
-    batch_finish<W>(d, s);
+    batch_finish<W>(d, f);
 }
 
 // (P)CG start: r = -g - q, p = z = M^-1 r with the Jacobi preconditioner M = (1 + lambda) D
@@ -244,7 +254,7 @@ __global__ void kb_cg_start(DotArgs d, const float2* __restrict__ g, float2* __r
             frr += brdot(ri, ri);
         }
     }
-    double s[2] = {frz, frr};
+    const float s[2] = {frz, frr};
     batch_finish<2>(d, s);
 }
 
@@ -272,7 +282,7 @@ __global__ void kb_cg_update(DotArgs d, float2* __restrict__ x, float2* __restri
             frz += dsc ? rr / (l1 * sc.D[i]) : rr;
         }
     }
-    double s[2] = {frz, frr};
+    const float s[2] = {frz, frr};
     batch_finish<2>(d, s);
 }
 
@@ -310,8 +320,7 @@ __global__ void kb_err_sums(DotArgs d, const float2* __restrict__ O, const float
             f[3] += rr.x * rr.x + rr.y * rr.y;
         }
     }
-    double s[4] = {f[0], f[1], f[2], f[3]};
-    batch_finish<4>(d, s);
+    batch_finish<4>(d, f);
 }
 
 }  // namespace

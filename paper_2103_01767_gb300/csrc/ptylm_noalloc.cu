@@ -61,7 +61,7 @@ k_loss_noalloc(const float2* __restrict__ O, const float2* __restrict__ P, const
     TeamCtx<G> c = team_setup<G>(tw_g);
     const float invS = 1.0f / G::S;
     const int ky = freq_ky<G>(c.tid);
-    double acc_l = 0.0, acc_d = 0.0;
+    SumPair acc[2] = {};   // l and dl^2 over this thread's pixels of all its positions
     float2 v[32];
     for (int k = blockIdx.x * G::TEAMS + c.team; k < K; k += gridDim.x * G::TEAMS) {
         const int2 rc = pos[k];
@@ -82,12 +82,11 @@ k_loss_noalloc(const float2* __restrict__ O, const float2* __restrict__ P, const
             sl += t.l;
             sd += t.dl * t.dl;
         }
-        acc_l += (double)sl;
-        acc_d += (double)sd;
+        pair_add(acc[0], sl);
+        pair_add(acc[1], sd);
         team_sync<G>();
     }
-    double sums[2] = {acc_l, acc_d};
-    grid_reduce<2>(sums, partials, counter, result, 0, OP_STORE, 1.0);
+    grid_reduce<2>(acc, partials, counter, result, 0, OP_STORE);
 }
 
 const void* kernel_for(int LS) {
