@@ -313,30 +313,39 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__
 
 // ---------------------------------------------------------------------------------------
 // Weight gradient: D_t[row][col] = sum over pixels p of A_t[row][p] B_t[col][p], one TMEM
-// accumulator per tap t.  One operand is the output gradient dy at the forward pass's output
-// pixels (shared by all taps), the other the tap-shifted input (copies as in the forward
-// pass).  Both are stored pixel-major with channels contiguous, i.e. MN-major operands; K is
-// the pixel index, 16 pixels (one row of the tile) per MMA.  A CTA runs over a strided
-// subset of the pixel tiles and writes its partial sums; k_wgrad_reduce adds them in a fixed
-// order.  Rows (or columns) beyond the real channel count read whatever lies next in shared
-// memory and are discarded.
+// accumulator of N columns per tap t.  One operand is the output gradient dy at the forward
+// pass's output pixels (shared by all taps), the other the tap-shifted input.  Both are stored
+// pixel-major with channels contiguous, i.e. MN-major operands; K is the pixel index, 16
+// pixels (one row of the tile) per MMA.  The input is loaded once per (parity) plane with the
+// columns the shifts reach, 18 pixels a row: in the no-swizzle layout a pixel is 16 bytes, so a
+// column shift is a descriptor offset like a row shift.  An MMA of 128 rows takes the tensor
+// pipe 64 cycles at N = 128, 48 at 64 and still 44 at 32, so a CTA holds as many columns as fit:
+// all nine taps up to N = 56, else the three taps of one kernel row with up to 128 columns
+// (nine taps of 32 columns before: layers 2-5 at batch 64 took 96, 212, 212 and 600 us).
+// A CTA runs over a strided subset of the pixel tiles and writes its partial sums;
+// k_wgrad_reduce adds them in a fixed order.  Rows beyond the real channel count read whatever
+// lies next in shared memory and are discarded.
 
 struct WgArgs {
     int tiles_x, tiles_y, phases, n_tiles, rows_px;
-    int w2;           // 0: A = dy (rows = output channels), B = input copies; 1: swapped
+    int w2;           // 0: A = dy (rows = output channels), B = input; 1: swapped
+    int taps;         // taps per CTA: 9, or 3 (one kernel row u = kind % 3)
+    int up;
     int g_real;       // dy chunk boxes per split
-    int x_real;       // input chunk boxes per copy and split
-    int n_copy, rows, N, c_tiles, Nc, tmem_cols, n_stage;
+    int x_real;       // input chunk boxes per plane and split
+    int planes, rows, N, c_tiles, tmem_cols, n_stage;
     int g_slot, x_slot, g_bytes, x_bytes, stage_bytes;
     int n_split;      // gridDim.x
-    int g_parity;     // 1: dy is read from its parity copy, plane = phase
-    Copy copy[6];
-    uint8_t grp[4][9][2];  // phase, tap -> copy, row offset
-    unsigned cmask[4];
+    int Co, Ci;
     float* part;
     unsigned* err;
     unsigned spin;
 };
+
+constexpr int kWgPx = 18, kWgPitch = kWgPx * 16;   // input pixels and bytes of a loaded row (8 channels)
+
+// floor((p + t - 1) / 2) for phase p in {0, 1} and tap t: the input pixel a tap of an upsampling layer reads
+__device__ __forceinline__ int tap_shift(int p, int t) { return (p + t + 1) / 2 - 1; }
 
 struct WgParams {
     CUtensorMap gmap[2];  // dy (or its parity copy): hi, lo
@@ -350,17 +359,28 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tc(const __grid_constant_
     __shared__ uint64_t full[kMaxStage], empty[kMaxStage], done;
     __shared__ uint32_t tbase;
     __shared__ int abort_flag, issued, consumed;
+    __shared__ uint32_t tap_at[4][9];   // phase, tap: offset of its input pixels in a stage, 16-byte units
     const WgArgs& a = p.a;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int split = blockIdx.x, kind = blockIdx.y;
     const int S = a.n_stage;
-    int o0, c0;
-    if (a.w2) {
-        c0 = kind * 128;
-        o0 = 0;
-    } else {
-        o0 = (kind / a.c_tiles) * 128;
-        c0 = (kind % a.c_tiles) * a.Nc;
+    const int u0 = a.taps == 3 ? kind % 3 : -1;            // the kernel row, -1: all
+    const int tile_kind = a.taps == 3 ? kind / 3 : kind;
+    const int mt = tile_kind / a.c_tiles, nt = tile_kind % a.c_tiles;
+    const int o0 = a.w2 ? nt * a.N : mt * 128, c0 = a.w2 ? mt * 128 : nt * a.N;
+    for (int i = threadIdx.x; i < a.phases * a.taps; i += kThreads) {
+        const int ph = i / a.taps, t = i % a.taps, u = a.taps == 3 ? u0 : t / 3, v = t % 3;
+        int plane, row, col;
+        if (a.up) {
+            plane = 0;
+            row = a.taps == 3 ? 0 : tap_shift(ph >> 1, u) + 1;
+            col = tap_shift(ph & 1, v) + 1;
+        } else {
+            plane = (a.taps == 3 ? 0 : 2 * (u != 1)) + (v != 1);
+            row = a.taps == 3 ? 0 : (u == 0 ? 0 : 1);
+            col = v == 0 ? 0 : 1;
+        }
+        tap_at[ph][t] = (uint32_t)(a.g_bytes + plane * a.x_real * a.x_slot + row * kWgPitch + col * 16) >> 4;
     }
     const int per_phase = a.tiles_x * a.tiles_y;
 
@@ -399,27 +419,26 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tc(const __grid_constant_
                     break;
                 }
                 if (*(volatile int*)&abort_flag) break;
-                const unsigned cm = a.cmask[ph];
-                uint32_t bytes = (uint32_t)(2 * a.g_real * a.g_slot);
-                for (int j = 0; j < a.n_copy; ++j)
-                    if (cm >> j & 1) bytes += (uint32_t)(2 * a.x_real * a.x_slot);
+                const uint32_t bytes = (uint32_t)(2 * (a.g_real * a.g_slot + a.planes * a.x_real * a.rows * kWgPitch));
                 const uint32_t st = sbase + s * a.stage_bytes;
                 const uint32_t fb = smem_u32(&full[s]);
                 bar_expect_tx(fb, bytes);
+                // first input row: all nine taps start one row up, one kernel row at its own
+                const int row0 = u0 < 0 ? a0 - 1 : a0 + (a.up ? tap_shift(ph >> 1, u0) : (u0 == 0 ? -1 : 0));
                 for (int sp = 0; sp < 2; ++sp) {
                     for (int q = 0; q < a.g_real; ++q) {
                         const int chunk = (o0 >> 3) + q;
                         tma_load_4d(st + (uint32_t)((sp * a.g_real + q) * a.g_slot), &p.gmap[sp], b0 * 8, a0,
-                                    a.g_parity ? 4 * chunk + ph : chunk, nimg, fb);
+                                    a.up ? 4 * chunk + ph : chunk, nimg, fb);
                     }
-                    for (int j = 0; j < a.n_copy; ++j) {
-                        if (!(cm >> j & 1)) continue;
-                        const Copy cp = a.copy[j];
-                        const uint32_t xb = st + (uint32_t)(a.g_bytes + ((sp * a.n_copy + j) * a.x_real) * a.x_slot);
+                    for (int pl = 0; pl < a.planes; ++pl) {
+                        // parity plane (qy, qx) of a stride-2 layer's input: pl = 2 qy + qx, or qx with qy = (u0 != 1)
+                        const int par = u0 < 0 ? pl : 2 * (u0 != 1) + pl;
+                        const uint32_t xb = st + (uint32_t)(a.g_bytes + ((sp * a.planes + pl) * a.x_real) * a.x_slot);
                         for (int q = 0; q < a.x_real; ++q) {
                             const int chunk = (c0 >> 3) + q;
-                            tma_load_4d(xb + (uint32_t)(q * a.x_slot), &p.xmap[sp], (b0 + cp.col) * 8, a0 + cp.row0,
-                                        cp.par < 0 ? chunk : 4 * chunk + cp.par, nimg, fb);
+                            tma_load_4d(xb + (uint32_t)(q * a.x_slot), &p.xmap[sp], (b0 - 1) * 8, row0,
+                                        a.up ? chunk : 4 * chunk + par, nimg, fb);
                         }
                     }
                 }
@@ -444,18 +463,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tc(const __grid_constant_
                 fence_after();
                 // operand offsets in the descriptors' 16-byte units, added to the stage's two
                 // descriptors (the issuing thread's time per MMA has to stay below the pipe's):
-                // the four wide layers' gradients at batch 64 1389 -> 1284 us in all
+                // the layers' gradients at batch 64 1389 -> 1284 us in all
                 const uint32_t st = sbase + s * a.stage_bytes;
                 const uint64_t gd0 = sdesc(st, 128u, (uint32_t)a.g_slot);
-                const uint64_t xd0 = sdesc(st + (uint32_t)a.g_bytes, 128u, (uint32_t)a.x_slot);
-                const uint32_t xlo = (uint32_t)(a.n_copy * a.x_real * a.x_slot) >> 4;  // hi -> lo half
+                const uint64_t xd0 = sdesc(st, 128u, (uint32_t)a.x_slot);
+                const uint32_t xlo = (uint32_t)(a.planes * a.x_real * a.x_slot) >> 4;  // hi -> lo half
                 const uint32_t glo = (uint32_t)(a.g_real * a.g_slot) >> 4;
-                for (int tap = 0; tap < 9; ++tap) {
+                for (int tap = 0; tap < a.taps; ++tap) {
                     const uint32_t d = tmem + (uint32_t)(tap * a.N);
-                    uint64_t gh = gd0, xh = xd0 + ((uint32_t)(a.grp[ph][tap][0] * a.x_real * a.x_slot + a.grp[ph][tap][1] * 256) >> 4);
+                    uint64_t gh = gd0, xh = xd0 + tap_at[ph][tap];
                     uint32_t acc = it > 0;
 #pragma unroll 4
-                    for (int k = 0; k < a.rows_px; ++k, gh += 16, xh += 16) {   // a row of 16 pixels is 256 bytes
+                    for (int k = 0; k < a.rows_px; ++k, gh += 16, xh += kWgPitch / 16) {   // a row of 16 dy pixels is 256 bytes
                         const uint64_t gl = gh + glo, xl = xh + xlo;
                         if (a.w2) {
                             mma_bf16(d, xh, gh, idesc, acc);
@@ -487,14 +506,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tc(const __grid_constant_
         const int row = 32 * warp + lane;
         const uint32_t lane_base = tmem + ((uint32_t)(32 * warp) << 16);
         const size_t blk = (size_t)kind * a.n_split + split;
-        for (int tap = 0; tap < 9; ++tap)
+        for (int tap = 0; tap < a.taps; ++tap)
             for (int cb = 0; cb < a.N; cb += 16) {
                 float v[16];
                 tmem_ld16(lane_base + (uint32_t)(tap * a.N + cb), v);
                 if (my_tiles == 0)
 #pragma unroll
                     for (int j = 0; j < 16; ++j) v[j] = 0.0f;
-                float4* dst = reinterpret_cast<float4*>(a.part + (((blk * 9 + tap) * 128 + row) * a.N + cb));
+                float4* dst = reinterpret_cast<float4*>(a.part + (((blk * a.taps + tap) * 128 + row) * a.N + cb));
 #pragma unroll
                 for (int q = 0; q < 4; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
             }
@@ -504,25 +523,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tc(const __grid_constant_
     if (warp == 0) tmem_dealloc(tmem, a.tmem_cols);
 }
 
-// dw[o][c][t] = sum_s part[kind][s][t][row][col] in split order
-__global__ void k_wgrad_reduce(const float* __restrict__ part, int Co, int Ci, int w2, int c_tiles, int Nc, int N,
+// dw[o][c][t] = sum_s part[kind][s][t][row][col] in split order; consecutive threads take
+// consecutive columns (blockIdx.y = kind)
+__global__ void k_wgrad_reduce(const float* __restrict__ part, int Co, int Ci, int w2, int taps, int c_tiles, int N,
                                int n_split, float* __restrict__ dw) {
-    const int total = Co * Ci * 9;
+    const int kind = blockIdx.y, total = taps * 128 * N;
+    const int tile_kind = taps == 3 ? kind / 3 : kind, mt = tile_kind / c_tiles, nt = tile_kind % c_tiles;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const int t = i % 9, c = (i / 9) % Ci, o = i / (9 * Ci);
-        int kind, row, col;
-        if (w2) {
-            kind = c / 128;
-            row = c % 128;
-            col = o;
-        } else {
-            kind = (o / 128) * c_tiles + c / Nc;
-            row = o % 128;
-            col = c % Nc;
-        }
+        const int col = i % N, row = (i / N) & 127, t = (taps == 3 ? 3 * (kind % 3) : 0) + i / (128 * N);
+        const int o = w2 ? nt * N + col : mt * 128 + row, c = w2 ? mt * 128 + row : nt * N + col;
+        if (o >= Co || c >= Ci) continue;
+        const float* src = part + (size_t)kind * n_split * total + i;
         float s = 0.0f;
-        for (int q = 0; q < n_split; ++q) s += part[((((size_t)kind * n_split + q) * 9 + t) * 128 + row) * N + col];
-        dw[i] = s;
+#pragma unroll 8
+        for (int q = 0; q < n_split; ++q) s += src[(size_t)q * total];
+        dw[((size_t)o * Ci + c) * 9 + t] = s;
     }
 }
 
@@ -660,14 +675,14 @@ bool g_ready = false;
 int g_conv_dyn = 0, g_wg_dyn = 0;   // dynamic shared memory the two kernels may request
 int g_conv_half = 0;                // ... and k_conv_tc with two CTAs on an SM
 
-// map of one half (hi or lo) of a chunk-major tensor; box = 16 pixels x 8 channels x `rows`
+// map of one half (hi or lo) of a chunk-major tensor; box = `px` pixels x 8 channels x `rows`
 // rows of one chunk (one parity plane of a parity-split tensor: chunk coordinate 4 q + plane)
-bool enc_act(CUtensorMap* m, const __nv_bfloat16* base, const Act2& t, bool parity, int rows) {
+bool enc_act(CUtensorMap* m, const __nv_bfloat16* base, const Act2& t, bool parity, int rows, int px = 16) {
     const size_t es = sizeof(__nv_bfloat16);
     const int C8 = t.C / 8, H = parity ? t.H / 2 : t.H, W = parity ? t.W / 2 : t.W, planes = parity ? 4 : 1;
     cuuint64_t dims[4] = {(cuuint64_t)W * 8, (cuuint64_t)H, (cuuint64_t)C8 * planes, (cuuint64_t)t.N};
     cuuint64_t strides[3] = {(cuuint64_t)W * 8 * es, (cuuint64_t)H * W * 8 * es, (cuuint64_t)C8 * planes * H * W * 8 * es};
-    cuuint32_t box[4] = {128, (cuuint32_t)rows, 1, 1}, estr[4] = {1, 1, 1, 1};
+    cuuint32_t box[4] = {(cuuint32_t)px * 8, (cuuint32_t)rows, 1, 1}, estr[4] = {1, 1, 1, 1};
     return g_encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(base), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -949,35 +964,34 @@ struct WgPlan {
 cudaError_t plan_wgrad(WgPlan& pl, const TcLayer& L, const Act2* x, const Act2* dy, int n_img, int num_sms) {
     std::memset(&pl, 0, sizeof pl);
     WgArgs& a = pl.prm.a;
-    a.w2 = L.Co <= 16 ? 1 : 0;
+    a.up = L.up;
+    a.Co = L.Co;
+    a.Ci = L.Ci;
+    // the 128 rows of an MMA go to the side that fills them
+    a.w2 = L.Co <= 16 || (L.Co < 128 && L.Ci >= 128) ? 1 : 0;
     a.phases = L.up ? 4 : 1;
     const int S = L.up ? L.Hin : L.Hout();   // per-phase output sub-lattice side
-    a.n_copy = L.up ? 3 : 6;
-    if (a.w2) {
-        a.N = (L.Co + 15) / 16 * 16;
-        a.g_real = (L.Co + 7) / 8;
-        a.x_real = std::min(16, L.Ci / 8);
-        a.c_tiles = 1;
-        a.Nc = 0;
-    } else {
-        a.Nc = L.Ci_pad >= 32 ? 32 : 16;
-        a.N = a.Nc;
-        a.g_real = std::min(16, L.Co / 8);
-        a.x_real = a.Nc / 8;
-        a.c_tiles = L.Ci_pad / a.Nc;
-    }
-    const int kinds = a.w2 ? (L.Ci + 127) / 128 : ((L.Co + 127) / 128) * a.c_tiles;
-    if (9 * a.N > 512) return cudaErrorInvalidConfiguration;
-    a.tmem_cols = pow2_cols(9 * a.N);
+    const int cols = a.w2 ? (L.Co + 15) / 16 * 16 : L.Ci_pad;
+    a.N = 16;
+    for (int n = 16; n <= std::min(128, cols); n += 16)
+        if (cols % n == 0) a.N = n;
+    a.taps = 9 * a.N <= 512 ? 9 : 3;
+    a.c_tiles = cols / a.N;
+    const int g_ch = a.w2 ? a.N : std::min(128, L.Co), x_ch = a.w2 ? std::min(128, L.Ci) : a.N;
+    a.g_real = std::min((L.Co + 7) / 8, g_ch / 8);
+    a.x_real = x_ch / 8;
+    const int kinds = ((a.w2 ? L.Ci : L.Co) + 127) / 128 * a.c_tiles * (9 / a.taps);
+    a.tmem_cols = pow2_cols(a.taps * a.N);
+    a.planes = L.up ? 1 : a.taps == 9 ? 4 : 2;
     // pixel rows per stage: 8 if two stages fit, else 4
     const int budget = g_wg_dyn - 1024;
     for (int rp = 8; rp >= 4; rp -= 4) {
         a.rows_px = rp;
-        a.rows = rp + (L.up ? 2 : 1);
+        a.rows = rp + (a.taps == 3 ? 0 : L.up ? 2 : 1);
         a.g_slot = rp * 16 * 16;
-        a.x_slot = a.rows * 256;
+        a.x_slot = (a.rows * kWgPitch + 127) / 128 * 128;   // a TMA load's destination: 128-byte aligned
         a.g_bytes = 2 * a.g_real * a.g_slot;
-        a.x_bytes = 2 * a.n_copy * a.x_real * a.x_slot;
+        a.x_bytes = 2 * a.planes * a.x_real * a.x_slot;
         a.stage_bytes = a.g_bytes + a.x_bytes;
         // rows / columns beyond the real channels read on into the next 16 slots at most
         const int tail = 16 * std::max(a.g_slot, a.x_slot);
@@ -989,33 +1003,6 @@ cudaError_t plan_wgrad(WgPlan& pl, const TcLayer& L, const Act2* x, const Act2* 
     a.tiles_x = S / 16;
     a.n_tiles = n_img * a.phases * a.tiles_x * a.tiles_y;
     a.n_split = std::max(1, std::min(a.n_tiles, num_sms / kinds));
-    for (int j = 0; j < a.n_copy; ++j) {
-        if (L.up) a.copy[j] = Copy{-1, (int8_t)(j - 1), -1};
-        else {
-            const int dxv[3] = {0, -1, 0}, qxv[3] = {0, 1, 1};
-            a.copy[j] = Copy{-1, (int8_t)dxv[j % 3], (int8_t)(2 * (j / 3) + qxv[j % 3])};
-        }
-    }
-    a.g_parity = L.up ? 1 : 0;
-    for (int ph = 0; ph < a.phases; ++ph) {
-        unsigned m = 0;
-        for (int u = 0; u < 3; ++u)
-            for (int v = 0; v < 3; ++v) {
-                int cp, ro;
-                if (L.up) {
-                    cp = half_shift(ph & 1, v) + 1;
-                    ro = half_shift(ph >> 1, u) + 1;
-                } else {
-                    const int qy = u == 1 ? 0 : 1, dyv = u == 0 ? -1 : 0, var = v == 1 ? 0 : (v == 0 ? 1 : 2);
-                    cp = qy * 3 + var;
-                    ro = dyv + 1;
-                }
-                a.grp[ph][3 * u + v][0] = (uint8_t)cp;
-                a.grp[ph][3 * u + v][1] = (uint8_t)ro;
-                m |= 1u << cp;
-            }
-        a.cmask[ph] = m;
-    }
     if (x && dy) {
         // up layers read dy by parity planes (its parity copy), stride-2 layers by plain rows;
         // the input x of a stride-2 layer is read by parity planes, of an up layer by plain rows
@@ -1023,7 +1010,8 @@ cudaError_t plan_wgrad(WgPlan& pl, const TcLayer& L, const Act2* x, const Act2* 
         const __nv_bfloat16* ghi = L.up ? dy->phi : dy->hi;
         const __nv_bfloat16* glo = L.up ? dy->plo : dy->lo;
         if (!enc_act(&pl.prm.gmap[0], ghi, *dy, L.up != 0, a.rows_px) || !enc_act(&pl.prm.gmap[1], glo, *dy, L.up != 0, a.rows_px) ||
-            !enc_act(&pl.prm.xmap[0], x->hi, *x, x->par != 0, a.rows) || !enc_act(&pl.prm.xmap[1], x->lo, *x, x->par != 0, a.rows))
+            !enc_act(&pl.prm.xmap[0], x->hi, *x, x->par != 0, a.rows, kWgPx) ||
+            !enc_act(&pl.prm.xmap[1], x->lo, *x, x->par != 0, a.rows, kWgPx))
             return cudaErrorInvalidValue;
     }
     pl.grid = dim3(a.n_split, kinds, 1);
@@ -1039,7 +1027,7 @@ size_t tc_wgrad_workspace(const TcLayer& L, int N, int num_sms) {
     if (tc_prepare() != cudaSuccess) return 0;
     static WgPlan pl;
     if (plan_wgrad(pl, L, nullptr, nullptr, N, num_sms) != cudaSuccess) return 0;
-    return (size_t)pl.grid.x * pl.grid.y * 9 * 128 * pl.prm.a.N;
+    return (size_t)pl.grid.x * pl.grid.y * pl.prm.a.taps * 128 * pl.prm.a.N;
 }
 
 cudaError_t tc_conv_wgrad(const TcLayer& L, const Act2& x, const Act2& dy, float* ws, float* dw, unsigned* err,
@@ -1054,9 +1042,8 @@ cudaError_t tc_conv_wgrad(const TcLayer& L, const Act2& x, const Act2& dy, float
     a.spin = spin;
     k_wgrad_tc<<<pl.grid, kThreads, pl.smem, st>>>(pl.prm);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const int total = L.Co * L.Ci * 9;
-    k_wgrad_reduce<<<std::max(1, std::min(4 * num_sms, (total + 255) / 256)), 256, 0, st>>>(
-        ws, L.Co, L.Ci, a.w2, a.c_tiles, a.Nc, a.N, a.n_split, dw);
+    k_wgrad_reduce<<<dim3((a.taps * 128 * a.N + 255) / 256, pl.grid.y), 256, 0, st>>>(ws, L.Co, L.Ci, a.w2, a.taps,
+                                                                                    a.c_tiles, a.N, a.n_split, dw);
     return cudaGetLastError();
 }
 
