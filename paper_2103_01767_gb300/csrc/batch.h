@@ -24,7 +24,8 @@ struct BatchProblem {
 // problem's probe side S and values per thread E (16, 4 and 1 for S = 32, 64, 128 with
 // E = 32; 8 and 2 for S = 32, 64 with E = 16).
 struct BatchItem {
-    int prob, k0, per_team, pad;
+    int prob, k0, per_team;
+    int run_end;          // index of the first later item that belongs to another problem
 };
 
 struct BatchArgs {

@@ -170,7 +170,10 @@ __device__ __forceinline__ void batch_item(const BatchArgs& a, const BatchProble
 }
 
 // The persistent scheduler: take items until none are left, then let the last CTA reset
-// the counters.
+// the counters.  Thread 0 fetches the next item's index while the CTA works on the present
+// one, except near the end, where an item held by a busy CTA would delay the launch.  At an
+// item of a masked-out problem it moves the counter past the rest of that problem's run of
+// items, so that launches with few problems left do not go through all the others' items.
 template <int KIND>
 __global__ void __launch_bounds__(BATCH_THREADS, 1) k_batch(BatchArgs a) {
     extern __shared__ float4 dyn_smem_f4[];
@@ -178,14 +181,21 @@ __global__ void __launch_bounds__(BATCH_THREADS, 1) k_batch(BatchArgs a) {
     float2* smem = tw + kBatchTwWords;
     __shared__ int s_item;
     batch_fill_twiddles(tw, a.tw);
+    int ahead = -1;   // thread 0: an index fetched early, or -1
     for (;;) {
-        if (threadIdx.x == 0) s_item = (int)atomicAdd(a.work, 1u);
+        if (threadIdx.x == 0) {
+            int idx = ahead >= 0 ? ahead : (int)atomicAdd(a.work, 1u);
+            while (a.active && idx < a.n_items && !a.active[a.items[idx].prob]) {
+                atomicMax(a.work, (unsigned)a.items[idx].run_end);
+                idx = (int)atomicAdd(a.work, 1u);
+            }
+            s_item = idx;
+            ahead = idx + 2 * (int)gridDim.x < a.n_items ? (int)atomicAdd(a.work, 1u) : -1;
+        }
         __syncthreads();  // also orders the twiddle stores before the first item
         const int idx = s_item;
-        __syncthreads();
         if (idx >= a.n_items) break;
         const BatchItem it = a.items[idx];
-        if (a.active && !a.active[it.prob]) continue;
         const BatchProblem p = a.probs[it.prob];
         switch (p.LS * 8 + p.LE) {
             case 5 * 8 + 5: batch_item<KIND, Geo<5, 5>>(a, p, it, smem, tw); break;

@@ -11,7 +11,10 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/ptylm.h"
@@ -216,6 +219,8 @@ __global__ void k_poisson_fmin(const float* __restrict__ y, long n, double* part
 // 304 slots of 64 x 64.)
 __global__ void __launch_bounds__(1024) k_probe_reduce(const float2* __restrict__ part, int slots, int M,
                                                        float2* __restrict__ out, int accumulate) {
+    griddep_launch();
+    griddep_wait();   // the product or gradient that fills `part`
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int m = blockIdx.x * 32 + lane;   // M is a multiple of 32
     __shared__ float2 val[2][32][32];
@@ -539,7 +544,10 @@ static bool joint(const ptylm_ctx* c) { return c->d.joint != 0; }
 // the teams that had a position (team s starts with position s).
 static ptylm_status probe_reduce(ptylm_ctx* c, int kid, float2* out, bool accumulate) {
     const int slots = std::min(c->grid[kid] * cta_teams(c->LS, c->LE), c->d.K);
-    k_probe_reduce<<<c->M / 32, 1024, 0, c->stream>>>(c->probe_part, slots, c->M, out, accumulate ? 1 : 0);
+    const float2* part = c->probe_part;
+    int M = c->M, acc = accumulate ? 1 : 0;
+    void* args[] = {&part, (void*)&slots, &M, &out, &acc};
+    CUDA_TRY(launch_dependent((const void*)k_probe_reduce, dim3(M / 32), dim3(1024), args, 0, c->stream));
     return vec_launched(c);
 }
 
@@ -728,6 +736,33 @@ static ptylm_status op_ggn_diag(ptylm_ctx* c, float* D, double floor_rel) {
     return PTYLM_OK;
 }
 
+// Whether a 16-CTA cluster of `fn` can be resident on `device` (asked once per kernel and
+// device: the answer does not change, and asking takes as long as a small lm_init).
+static bool cluster_cg_usable(const void* fn, int device) {
+    static std::mutex mutex;
+    static std::map<std::pair<const void*, int>, bool> known;
+    std::lock_guard<std::mutex> lock(mutex);
+    auto it = known.find({fn, device});
+    if (it != known.end()) return it->second;
+    bool ok = false;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = kClusterCtas;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.gridDim = dim3(kClusterCtas);
+        cfg.blockDim = dim3(kClusterThreads);
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        ok = cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters > 0;
+    }
+    cudaGetLastError();
+    known[{fn, device}] = ok;
+    return ok;
+}
+
 // ---------------------------------------------------------------------------------------
 // C-ABI
 // ---------------------------------------------------------------------------------------
@@ -843,12 +878,14 @@ ptylm_status lm_init(ptylm_ctx** out, const ptylm_desc* desc, const int32_t* pos
         cudaGetLastError();
         return bail(fail(PTYLM_ERR_CUDA, "no usable CUDA device"));
     }
-    // FFT tile: 32 values per thread, or 16 for sides 32 and 64 when teams of S^2/32 threads
-    // would fill less than half of the GPU's thread slots (few positions): twice the threads
-    // per patch halve each position's dependent chain of FFT passes
+    // FFT tile: 16 values per thread for side 64 and for blind problems of side 32, where it is
+    // the faster one over the whole range of K (64^2, 1900 positions, 16 / 32 values: product 45.7 /
+    // 50.8 us, blind product 65.8 / 83.5, loss 29.5 / 34.6; 32^2 blind, 8000: 74.7 / 105 us); for
+    // other 32^2 problems while teams of S^2/32 threads would fill less than half of the GPU's
+    // thread slots (product at 3000 positions 20.6 / 20.7 us, at 8000 41.2 / 37.0).
     if (d.values_per_thread == 16) c->LE = 4;
     else if (d.values_per_thread == 32) c->LE = 5;
-    else c->LE = (LS <= 6 && (long)d.K * (c->M / 32) < (long)c->num_sms * 1024) ? 4 : 5;
+    else c->LE = LS == 6 || (LS == 5 && (d.joint || (long)d.K * (c->M / 32) < (long)c->num_sms * 1024)) ? 4 : 5;
     const int teams = cta_teams(LS, c->LE);
     for (int kid = 0; kid < KID_COUNT; ++kid) {
         int per_sm = 0;
@@ -879,19 +916,7 @@ ptylm_status lm_init(ptylm_ctx** out, const ptylm_desc* desc, const int32_t* pos
         // One cluster for short vectors.  (The three-launch form then runs on as many CTAs, whose
         // partial sums have to fit.)
         const void* fn = c->coop_grid > 0 && c->partials_cap >= kClusterCtas ? cg_cluster_kernel(c->L) : nullptr;
-        if (fn && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-            cudaLaunchConfig_t cfg = {};
-            cudaLaunchAttribute at;
-            at.id = cudaLaunchAttributeClusterDimension;
-            at.val.clusterDim.x = kClusterCtas;
-            at.val.clusterDim.y = at.val.clusterDim.z = 1;
-            cfg.gridDim = dim3(kClusterCtas);
-            cfg.blockDim = dim3(kClusterThreads);
-            cfg.attrs = &at;
-            cfg.numAttrs = 1;
-            int clusters = 0;
-            if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters > 0) c->cluster_cg = fn;
-        }
+        if (fn && cluster_cg_usable(fn, c->device)) c->cluster_cg = fn;
         cudaGetLastError();
     }
 

@@ -443,6 +443,8 @@ std::vector<BatchItem> build_items(const ptylm_batch* bt, int order, int per_tea
             for (int b = 0; b < bt->B; ++b)
                 if (i < per[b].size()) out.push_back(per[b][i]);
     }
+    for (int i = (int)out.size() - 1; i >= 0; --i)
+        out[i].run_end = i + 1 < (int)out.size() && out[i + 1].prob == out[i].prob ? out[i + 1].run_end : i + 1;
     return out;
 }
 
