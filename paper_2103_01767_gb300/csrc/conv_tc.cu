@@ -1,29 +1,34 @@
 // conv_tc.cu -- tensor-core 3x3 convolutions of the learned initialisation (see conv_tc.h).
 //
-// Implicit GEMM.  A CTA owns a tile of 8 x 16 points of an output sub-lattice (the output
-// grid itself, or one parity class of it), i.e. 128 GEMM rows = 128 TMEM lanes, and up to four
-// such accumulators ("phases") of N columns each.  The K loop runs over input channels, 16 per
-// pipeline stage.  Per stage a TMA producer thread loads
-//   * a few "copies" of the input: boxes of (8 channels) x (16 columns) x (rows) from the map or
-//     one of its parity planes, each with its own column shift (every box row is 256
-//     contiguous bytes of the chunk-major layout); a tap's
-//     operand is a copy started `row` rows down (the canonical no-swizzle K-major layout makes
-//     a row shift a plain descriptor offset, so one copy serves the three taps of a column);
-//     out-of-range coordinates fill zeros, which is the convolution's zero padding;
+// Implicit GEMM.  A tile is 16 x 8 points of an output sub-lattice (the output grid itself, or
+// one parity class of it), i.e. 128 GEMM rows = 128 TMEM lanes, with up to four accumulators
+// ("phases") of N columns each.  A persistent CTA per SM runs over tiles in three roles: one
+// thread loads, one issues the MMAs, eight warps write the results; the accumulators are
+// double buffered, so a tile's epilogue overlaps the next tile's MMAs.  The K loop runs over
+// input channels, 16 per pipeline stage.  Per stage the TMA producer loads
+//   * the input: boxes of (8 channels) x (9 or 10 columns) x (17 or 18 rows) from the map or its
+//     parity planes.  In the canonical no-swizzle K-major layout a pixel's 8 channels are 16
+//     bytes and 8 pixels a core matrix, so with 8-pixel tile rows the box row is the stride
+//     between core matrices and a tap's row and column shift are a plain descriptor offset: one
+//     box serves all taps.  Out-of-range coordinates fill zeros, the convolution's zero padding;
 //   * the bfloat16 weights of all nine taps for those 16 channels (18 contiguous bulk copies);
-// and one MMA thread issues, per (phase, tap) group and per split (hi, lo), a 128 x N x 16
+// and the MMA thread issues, per (phase, tap) group and per split (hi, lo), a 128 x N x 16
 // tcgen05.mma into the phase's accumulator.  Mbarrier rings (full / empty) pipeline the stages.
 //
 // Layer forms (s: stride-2 layer, u: upsampling layer):
-//   forward s:  output (a, b) reads input (2a+u-1, 2b+v-1): six copies from the four parity
-//               views of the input (column shift 0 or -1);
+//   forward s:  output (a, b) reads input (2a+u-1, 2b+v-1): the four parity planes;
 //   forward u:  four phases (py, px) of the output (2a+py, 2b+px) read the low-resolution
-//               input at (a + floor((py+u-1)/2), b + floor((px+v-1)/2)): three copies;
+//               input at (a + floor((py+u-1)/2), b + floor((px+v-1)/2));
 //   input gradient s: four phases (qy, qx) of the input grid, (2a'+qy, 2b'+qx), collect dy at
 //               (a' + e, b' + f), e, f in {0, 1}, from the taps with matching parity;
 //   input gradient u: a stride-1 correlation of dy at full resolution whose 2 x 2 sums (taken
-//               with warp shuffles: a warp holds two full rows of the tile) give the gradient
+//               with warp shuffles: a warp holds four rows of the tile) give the gradient
 //               of the low-resolution input.
+//
+// Forward pass of 225 patterns (widths 64/128/256), layers 1-5: 111, 71, 73, 145, 208 us; with
+// one CTA per tile, 16-pixel tile rows, a copy of the input per column shift and operands
+// moved to uniform registers MMA by MMA 179, ~100, 115, 294, ~343 us.  Layers 4 and 5 run at
+// about 0.75 of the rate their MMAs allow, 1-3 are bound by their epilogues and loads.
 // The weight gradient is a GEMM over pixels with MN-major operands (k_wgrad_tc).
 #include "conv_tc.h"
 
@@ -41,8 +46,10 @@ namespace {
 using namespace tc;
 
 constexpr int kThreads = 128;
+constexpr int kEpiThreads = 256;      // epilogue: two groups of four warps, which share the 128 lanes
+constexpr int kConvThreads = kEpiThreads + 64;   // ... the TMA warp, the MMA warp
 constexpr int kMaxStage = 8;
-constexpr int kMaxCopy = 8;
+constexpr int kMaxCopy = 4;
 constexpr int kMaxGroup = 36;
 constexpr int kSmemLimit = 232448;    // shared memory a CTA may use (static + dynamic)
 constexpr int kOneCtaPerSm = 120 * 1024;  // dynamic request that leaves no room for a second CTA
@@ -54,17 +61,17 @@ struct Copy {
     int8_t par;        // parity plane of a parity-split map, -1 for a plain map
 };
 struct Group {
-    uint8_t phase, copy, row, tap;
+    uint8_t phase, copy, row, col, tap;
 };
 
 struct ConvArgs {
-    int tiles_x, tiles_y;  // 8 x 16 tiles per image
-    int n_copy, split, rows, ksteps, N, P, tmem_cols, n_stage;
-    int a_slot;       // bytes of one (copy, chunk) box: rows * 256
+    int tiles_x, tiles_y;  // 16 x 8 (rows x columns) tiles per image
+    int n_img, pgroups, n_zt;   // tiles: images x space, phase groups, column (channel) tiles
+    int n_copy, split, rows, px, ksteps, N, P, n_acc, tmem_cols, n_stage;
+    int a_slot;       // bytes of one (copy, chunk) box, rows * px * 16 rounded up to 128
     int a_bytes;      // A bytes of a stage: split * n_copy * 2 * a_slot
     int stage_bytes;  // a_bytes + 2 * 9 * N * 16
     int gstart[5];    // groups sorted by phase: phase p owns [gstart[p], gstart[p+1])
-    unsigned cmask[4];  // copies used per phase group
     Copy copy[kMaxCopy];
     Group group[kMaxGroup];
     int mode, osy, osx;
@@ -91,16 +98,11 @@ struct ConvArgs {
 struct ConvParams {
     CUtensorMap amap[2];  // the input tensor: hi, lo
     ConvArgs a;
+    uint4 mma[2 * kMaxGroup];   // per group and split: offsets of A and B in a stage (16-byte units), column, accumulate
 };
 
 __device__ __forceinline__ unsigned char* align1024(unsigned char* p) {
     return reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~uintptr_t(1023));
-}
-
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
 }
 
 // 16 channels from ch0 of pixel (y, x) into the output pair (and its parity copy)
@@ -113,20 +115,118 @@ __device__ __forceinline__ void store_out16(const ConvArgs& a, int n, int y, int
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__ ConvParams p) {
+// the epilogue warps only
+__device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
+
+// One tile's accumulators (at `lane_base`, this warp's TMEM lanes) through the layer's epilogue.
+// Warps w and w + 4 hold the same 128 pixels and take 32 columns each of every 64; what a step
+// reads from memory (the ReLU mask) is fetched before its accumulators are waited for.  With
+// four warps and the mask read inside the step the input gradients of a batch of 64 took 223,
+// 136, 76 and 128 us, now 138, 83, 52 and 82.
+__device__ __forceinline__ void conv_epilogue(const ConvArgs& a, uint32_t lane_base, int n, int a0, int b0, int pg, int o0,
+                                              size_t part, float (*red)[256]) {
+    const int warp = (threadIdx.x >> 5) & 3, grp = threadIdx.x >> 7, lane = threadIdx.x & 31;
+    const int r = (threadIdx.x & 127) >> 3, c = threadIdx.x & 7;
+    const bool pooled = a.mode == EPI_POOL, writer = !pooled || ((r | c) & 1) == 0;
+    if (a.mode >= EPI_BWD) {
+        for (int i = threadIdx.x; i < 4 * 256; i += kEpiThreads) (&red[0][0])[i] = 0.0f;
+        epilogue_sync();
+    }
+    for (int ph = 0; ph < a.P; ++ph) {
+        const int phase = pg * a.P + ph;
+        const int oy = a.osy * (a0 + r) + a.opy[phase], ox = a.osx * (b0 + c) + a.opx[phase];
+        const int py = pooled ? (a0 + r) >> 1 : oy, px = pooled ? (b0 + c) >> 1 : ox;
+        auto columns16 = [&](float (&v)[16], const uint4 (&mk)[4], int cb) {
+            const int ch0 = o0 + cb;
+            if (a.mode == EPI_HIDDEN) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    v[j] += __ldg(a.bias + ch0 + j);
+                    if (a.relu) v[j] = fmaxf(v[j], 0.0f);
+                }
+                store_out16(a, n, oy, ox, ch0, v);
+            } else if (a.mode == EPI_LAST) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (ch0 + j < a.oC)
+                        a.out32[(((size_t)n * a.oC + ch0 + j) * a.oH + oy) * a.oW + ox] = v[j] + a.bias[ch0 + j];
+            } else {
+                if (pooled) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        v[j] += __shfl_xor_sync(0xffffffffu, v[j], 1);
+                        v[j] += __shfl_xor_sync(0xffffffffu, v[j], 8);
+                    }
+                }
+                if (writer) {
+                    bool m[16];
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) mask8(mk[2 * q], mk[2 * q + 1], m + 8 * q);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) v[j] = m[j] ? v[j] : 0.0f;
+                    store_out16(a, n, py, px, ch0, v);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) v[j] = 0.0f;
+                }
+                // column sums over the warp: each exchange halves the columns a lane carries on
+                // (16 shuffles, against 80 for sixteen separate trees)
+#pragma unroll
+                for (int half = 8; half >= 1; half >>= 1) {
+                    const bool up = lane & (2 * half);
+#pragma unroll
+                    for (int j = 0; j < half; ++j) {
+                        const float keep = up ? v[j + half] : v[j], send = up ? v[j] : v[j + half];
+                        v[j] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * half);
+                    }
+                }
+                v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+                if (!(lane & 1)) red[warp][cb + (lane >> 1)] += v[0];
+            }
+        };
+        for (int cb = 32 * grp; cb < a.N; cb += 64) {
+            float w[2][16];
+            uint4 mk[2][4];
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (cb + 16 * q < a.N) tmem_ld16_start(lane_base + (uint32_t)(ph * a.N + cb + 16 * q), w[q]);
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    mk[q][2 * h] = mk[q][2 * h + 1] = make_uint4(0, 0, 0, 0);
+                    if (a.mode >= EPI_BWD && writer && cb + 16 * q < a.N) {
+                        const size_t o = chunk_at(a.m_par, a.oC >> 3, a.oH, a.oW, n, py, px, ((o0 + cb) >> 3) + 2 * q + h);
+                        mk[q][2 * h] = __ldg(reinterpret_cast<const uint4*>(a.m_hi + o));
+                        mk[q][2 * h + 1] = __ldg(reinterpret_cast<const uint4*>(a.m_lo + o));
+                    }
+                }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) tmem_ld_wait16(w[q]);
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (cb + 16 * q < a.N) columns16(w[q], mk[q], cb + 16 * q);
+        }
+    }
+    if (a.mode >= EPI_BWD) {
+        epilogue_sync();
+        for (int ch = threadIdx.x; ch < a.N; ch += kEpiThreads)
+            a.db_part[part * a.oC + o0 + ch] = red[0][ch] + red[1][ch] + red[2][ch] + red[3][ch];
+        epilogue_sync();   // before the next tile clears red
+    }
+}
+
+__global__ void __launch_bounds__(kConvThreads, 1) k_conv_tc(const __grid_constant__ ConvParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = align1024(smem_raw);
-    __shared__ uint64_t full[kMaxStage], empty[kMaxStage], done;
+    __shared__ uint64_t full[kMaxStage], empty[kMaxStage], acc_full[2], acc_empty[2], done;
     __shared__ uint32_t tbase;
-    __shared__ int abort_flag, issued, consumed;
+    __shared__ int abort_flag, epilogue_abort, issued, consumed;
     __shared__ float red[4][256];
-    __shared__ uint4 mma_list[2 * kMaxGroup];
     const ConvArgs& a = p.a;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int per_img = a.tiles_x * a.tiles_y;
-    const int n = blockIdx.x / per_img, t = blockIdx.x % per_img;
-    const int a0 = (t / a.tiles_x) * 8, b0 = (t % a.tiles_x) * 16;
-    const int pg = blockIdx.y, o0 = blockIdx.z * a.N;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int per_img = a.tiles_x * a.tiles_y, n_xt = per_img * a.n_img;
+    const int pg = blockIdx.y, total = n_xt * a.n_zt;   // channel tiles fastest: they share the input
     const int S = a.n_stage;
 
     if (warp == 0) tmem_alloc(smem_u32(&tbase), a.tmem_cols);
@@ -135,176 +235,147 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__
             bar_init(smem_u32(&full[s]), 1);
             bar_init(smem_u32(&empty[s]), 1);
         }
+        for (int s = 0; s < 2; ++s) {
+            bar_init(smem_u32(&acc_full[s]), 1);
+            bar_init(smem_u32(&acc_empty[s]), kEpiThreads / 32);
+        }
         bar_init(smem_u32(&done), 1);
         bar_fence_init();
         abort_flag = 0;
+        epilogue_abort = 0;
         issued = 0;
         consumed = 0;
-    }
-    for (int i = threadIdx.x; i < 4 * 256; i += kThreads) (&red[0][0])[i] = 0.0f;
-    const int g0 = a.gstart[pg * a.P], n_mma = (a.gstart[pg * a.P + a.P] - g0) * a.split;
-    for (int i = threadIdx.x; i < n_mma; i += kThreads) {
-        const Group gr = a.group[g0 + i / a.split];
-        const int sp = i % a.split, ph = gr.phase - pg * a.P;
-        const bool first = sp == 0 && g0 + i / a.split == a.gstart[gr.phase];
-        mma_list[i] = make_uint4((uint32_t)((sp * a.n_copy + gr.copy) * 2 * a.a_slot + gr.row * 256) >> 4,
-                                 (uint32_t)(gr.tap * a.N * 16) >> 4, (uint32_t)(ph * a.N), first ? 0u : 1u);
     }
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tmem = tbase;
-    const uint32_t sbase = smem_u32(smem);
-    const unsigned cmask = a.cmask[pg];
+    const uint32_t tmem = (uint32_t)uniform((int)tbase);
+    const uint32_t sbase = (uint32_t)uniform((int)smem_u32(smem));
+    volatile int* aborted = &abort_flag;
 
-    if (warp == 0) {
-        // TMA producer: lane 0 issues, the other lanes wait at the warp barrier
-        if (lane == 0) {
-            const int nb = min(a.N, a.wR - o0);   // weight rows present (the rest is never read into D)
-            uint32_t bytes = 18u * (uint32_t)nb * 16u;
-            for (int j = 0; j < a.n_copy; ++j)
-                if (cmask >> j & 1) bytes += (uint32_t)(a.split * 2 * a.a_slot);
-            int ks = 0;
-            for (; ks < a.ksteps; ++ks) {
-                const int s = ks % S, use = ks / S;
-                if (use > 0 && !bar_wait(smem_u32(&empty[s]), (use - 1) & 1, a.spin)) {
-                    atomicOr(a.err, 1u);
-                    abort_flag = 1;
-                    break;
-                }
-                if (*(volatile int*)&abort_flag) break;
-                const uint32_t st = sbase + s * a.stage_bytes;
-                const uint32_t fb = smem_u32(&full[s]);
-                bar_expect_tx(fb, bytes);
-                for (int sp = 0; sp < a.split; ++sp)
-                    for (int j = 0; j < a.n_copy; ++j) {
-                        if (!(cmask >> j & 1)) continue;
-                        const uint32_t dst = st + (uint32_t)((sp * a.n_copy + j) * 2 * a.a_slot);
-                        const Copy cp = a.copy[j];
-                        const int x = (b0 + cp.col) * 8, y = a0 + cp.row0;
+    if (warp == kEpiThreads / 32) {
+        if (elect_one()) {   // TMA producer
+            const uint32_t abytes = (uint32_t)(a.split * a.n_copy * 2 * a.rows * a.px * 16);
+            int it = 0, s = 0;
+            uint32_t par = 1;   // a fresh barrier's previous phase counts as complete
+            for (int t = blockIdx.x; t < total && !*aborted; t += gridDim.x) {
+                const int xt = t / a.n_zt, o0 = (t - xt * a.n_zt) * a.N;
+                const int n = xt / per_img, tt = xt - n * per_img, ty = tt / a.tiles_x;
+                const int a0 = ty * 16, b0 = (tt - ty * a.tiles_x) * 8;
+                const int nb = min(a.N, a.wR - o0);   // weight rows present (the rest is never read into D)
+                // a tap's weights of the stage's two chunks are contiguous when the tile holds all rows
+                const int wq = nb == a.wR && nb == a.N ? 1 : 2;
+                for (int ks = 0; ks < a.ksteps; ++ks, ++it) {
+                    const uint32_t st = sbase + s * a.stage_bytes, fb = smem_u32(&full[0]) + 8 * s;
+                    if (!bar_wait(smem_u32(&empty[0]) + 8 * s, par, a.spin)) {
+                        atomicOr(a.err, 1u);
+                        abort_flag = 1;
+                    }
+                    if (*aborted) break;
+                    bar_expect_tx(fb, abytes + 18u * (uint32_t)nb * 16u);
+                    for (int sp = 0; sp < a.split; ++sp)
+                        for (int j = 0; j < a.n_copy; ++j) {
+                            const uint32_t dst = st + (uint32_t)((sp * a.n_copy + j) * 2 * a.a_slot);
+                            const Copy cp = a.copy[j];
+                            const int x = (b0 + cp.col) * 8, y = a0 + cp.row0;
 #pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            const int chunk = 2 * ks + q;
-                            tma_load_4d(dst + q * a.a_slot, &p.amap[sp], x, y, cp.par < 0 ? chunk : 4 * chunk + cp.par, n, fb);
+                            for (int q = 0; q < 2; ++q) {
+                                const int chunk = 2 * ks + q;
+                                tma_load_4d(dst + q * a.a_slot, &p.amap[sp], x, y, cp.par < 0 ? chunk : 4 * chunk + cp.par, n, fb);
+                            }
                         }
-                    }
-                const uint32_t bdst = st + a.a_bytes;
-                for (int q = 0; q < 2; ++q)
-                    for (int t = 0; t < 9; ++t) {
-                        const __nv_bfloat16* src = a.wts + (((size_t)t * a.wK8 + 2 * ks + q) * a.wR + o0) * 8;
-                        bulk_load(bdst + (uint32_t)((q * 9 + t) * a.N * 16), src, (uint32_t)nb * 16u, fb);
-                    }
+                    const uint32_t bdst = st + a.a_bytes;
+                    for (int w = 0; w < 9; ++w)
+                        for (int q = 0; q < wq; ++q) {
+                            const __nv_bfloat16* src = a.wts + (((size_t)w * a.wK8 + 2 * ks + q) * a.wR + o0) * 8;
+                            bulk_load(bdst + (uint32_t)((2 * w + q) * a.N * 16), src, (uint32_t)nb * (wq == 1 ? 32u : 16u), fb);
+                        }
+                    if (++s == S) s = 0, par ^= 1u;
+                }
             }
-            issued = ks;
+            issued = it;
         }
         __syncwarp();
-    } else if (warp == 1) {
-        // MMA issuer: lane 0 issues, the other lanes wait at the warp barrier
-        if (lane == 0) {
-            // One thread feeds the tensor pipe, which takes an MMA every 44 (N <= 32), 48 (N = 64)
-            // or 64 cycles (N = 128; the shared-memory reads of A and B bound the smaller N).
-            // Building each MMA's descriptors from its group took that thread about 100 cycles;
-            // now every operand offset comes from mma_list, in the descriptors' 16-byte units.
-            // With two CTAs per SM (finish_plan) the layers of a 225-pattern forward pass went
-            // 429 (mean of layers 2 and 5), 146 and 332 us (3 and 4) -> 222, 115 and 294 us.
+    } else if (warp == kEpiThreads / 32 + 1) {
+        if (elect_one()) {
+            // MMA issuer.  The tensor pipe takes an MMA every 44 (N <= 32), 48 (N = 64) or 64 cycles
+            // (N = 128; the shared-memory reads of A and B bound the smaller N), so issuing one may
+            // cost no more: the operand offsets come from a table in the kernel's parameters, in the
+            // descriptors' 16-byte units, and everything they are added to is a loop counter, a
+            // parameter or a block index, which stays in uniform registers (tc_common.cuh).
             const uint32_t idesc = idesc_bf16(128, a.N, 0, 0);
-            int ks = 0;
-            for (; ks < a.ksteps; ++ks) {
-                const int s = ks % S, use = ks / S;
-                if (!bar_wait(smem_u32(&full[s]), use & 1, a.spin)) {
-                    atomicOr(a.err, 2u);
+            const int i0 = a.gstart[pg * a.P] * a.split, i1 = a.gstart[pg * a.P + a.P] * a.split;
+            int it = 0, s = 0, buf = 0;
+            uint32_t par = 0, apar = 1;
+            bool gone = false;
+            for (int t = blockIdx.x; t < total && !gone; t += gridDim.x) {
+                if (!bar_wait(smem_u32(&acc_empty[0]) + 8 * buf, apar, a.spin)) {
+                    atomicOr(a.err, 64u);
                     abort_flag = 1;
                     break;
                 }
                 fence_after();
-                const uint32_t st = sbase + s * a.stage_bytes;
-                const uint64_t ad0 = sdesc(st, (uint32_t)a.a_slot, 128u);
-                const uint64_t bd0 = sdesc(st + a.a_bytes, 9u * a.N * 16u, 128u);
-#pragma unroll 6
-                for (int i = 0; i < n_mma; ++i) {
-                    const uint4 m = mma_list[i];
-                    mma_bf16(tmem + m.z, ad0 + m.x, bd0 + m.y, idesc, m.w | (uint32_t)ks);
+                const uint32_t d0 = tmem + (uint32_t)(buf * a.P * a.N);
+                for (int ks = 0; ks < a.ksteps; ++ks, ++it) {
+                    if (!bar_wait(smem_u32(&full[0]) + 8 * s, par, a.spin)) {
+                        atomicOr(a.err, 2u);
+                        abort_flag = 1;
+                        gone = true;
+                        break;
+                    }
+                    fence_after();
+                    const uint32_t st = sbase + s * a.stage_bytes;
+                    const uint64_t ad0 = sdesc(st, (uint32_t)a.a_slot, (uint32_t)a.px * 16u);
+                    const uint64_t bd0 = sdesc(st + a.a_bytes, (uint32_t)a.N * 16u, 128u);
+#pragma unroll 4
+                    for (int i = i0; i < i1; ++i) {
+                        const uint4 m = p.mma[i];
+                        mma_bf16(d0 + m.z, ad0 + m.x, bd0 + m.y, idesc, m.w | (uint32_t)ks);
+                    }
+                    mma_commit(smem_u32(&empty[0]) + 8 * s);
+                    if (++s == S) s = 0, par ^= 1u;
                 }
-                mma_commit(smem_u32(&empty[s]));
+                mma_commit(smem_u32(&acc_full[0]) + 8 * buf);
+                if (++buf == a.n_acc) buf = 0, apar ^= 1u;
+                gone = gone || *aborted;
             }
-            consumed = ks;
+            consumed = it;
             mma_commit(smem_u32(&done));
         }
         __syncwarp();
+    } else {
+        int buf = 0;
+        uint32_t fpar = 0;
+        for (int t = blockIdx.x; t < total; t += gridDim.x) {
+            const int xt = t / a.n_zt, o0 = (t - xt * a.n_zt) * a.N;
+            const int n = xt / per_img, tt = xt % per_img;
+            // all epilogue warps leave together (the epilogue has barriers of its own): the flag they
+            // test is only written between the barrier at the end of a tile and the next one
+            const bool ok = bar_wait(smem_u32(&acc_full[buf]), fpar, a.spin);
+            if (!ok && lane == 0) {
+                atomicOr(a.err, 4u);
+                abort_flag = 1;
+            }
+            if (lane == 0 && *aborted) *(volatile int*)&epilogue_abort = 1;
+            epilogue_sync();
+            if (*(volatile int*)&epilogue_abort) break;
+            fence_after();
+            conv_epilogue(a, tmem + (uint32_t)(buf * a.P * a.N) + ((uint32_t)(32 * (warp & 3)) << 16), n, (tt / a.tiles_x) * 16,
+                          (tt % a.tiles_x) * 8, pg, o0, (size_t)pg * n_xt + xt, red);
+            fence_before();
+            __syncwarp();
+            if (lane == 0) bar_arrive(smem_u32(&acc_empty[buf]));
+            if (++buf == a.n_acc) buf = 0, fpar ^= 1u;
+            epilogue_sync();
+        }
     }
     const bool ok = bar_wait(smem_u32(&done), 0, a.spin);
     if (!ok && lane == 0) atomicOr(a.err, 4u);
     fence_after();
     __syncthreads();
-    const bool abort = *(volatile int*)&abort_flag || !ok;
-    if (abort && threadIdx.x == 0) {
+    if ((*aborted || !ok) && threadIdx.x == 0) {
         // let the copies still in flight land before the CTA's shared memory is released
-        for (int ks = consumed; ks < issued; ++ks) bar_wait(smem_u32(&full[ks % S]), (ks / S) & 1, a.spin);
-    }
-
-    if (!abort) {
-        const int i = 32 * warp + lane;
-        const int r = i >> 4, c = i & 15;
-        const uint32_t lane_base = tmem + ((uint32_t)(32 * warp) << 16);
-        for (int ph = 0; ph < a.P; ++ph) {
-            const int phase = pg * a.P + ph;
-            const int oy = a.osy * (a0 + r) + a.opy[phase], ox = a.osx * (b0 + c) + a.opx[phase];
-            for (int cb = 0; cb < a.N; cb += 16) {
-                float v[16];
-                tmem_ld16(lane_base + (uint32_t)(ph * a.N + cb), v);
-                const int ch0 = o0 + cb;
-                if (a.mode == EPI_HIDDEN) {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        v[j] += a.bias[ch0 + j];
-                        if (a.relu) v[j] = fmaxf(v[j], 0.0f);
-                    }
-                    store_out16(a, n, oy, ox, ch0, v);
-                } else if (a.mode == EPI_LAST) {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        if (ch0 + j < a.oC)
-                            a.out32[(((size_t)n * a.oC + ch0 + j) * a.oH + oy) * a.oW + ox] = v[j] + a.bias[ch0 + j];
-                } else {
-                    int py = oy, px = ox;
-                    bool writer = true;
-                    if (a.mode == EPI_POOL) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            v[j] += __shfl_xor_sync(0xffffffffu, v[j], 1);
-                            v[j] += __shfl_xor_sync(0xffffffffu, v[j], 16);
-                        }
-                        writer = ((r | c) & 1) == 0;
-                        py = (a0 + r) >> 1;
-                        px = (b0 + c) >> 1;
-                    }
-                    if (writer) {
-                        bool m[16];
-#pragma unroll
-                        for (int q = 0; q < 2; ++q)
-                            load_mask8(a.m_hi, a.m_lo, chunk_at(a.m_par, a.oC >> 3, a.oH, a.oW, n, py, px, (ch0 >> 3) + q),
-                                       m + 8 * q);
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) v[j] = m[j] ? v[j] : 0.0f;
-                        store_out16(a, n, py, px, ch0, v);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) v[j] = 0.0f;
-                    }
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float sum = warp_sum(v[j]);
-                        if (lane == 0) red[warp][cb + j] += sum;
-                    }
-                }
-            }
-        }
-        if (a.mode >= EPI_BWD) {
-            __syncthreads();
-            const size_t part = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
-            for (int ch = threadIdx.x; ch < a.N; ch += kThreads)
-                a.db_part[part * a.oC + o0 + ch] = red[0][ch] + red[1][ch] + red[2][ch] + red[3][ch];
-        }
+        for (int it = consumed; it < issued; ++it) bar_wait(smem_u32(&full[it % S]), (it / S) & 1, a.spin);
     }
     fence_before();
     __syncthreads();
@@ -321,7 +392,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__
 // column shift is a descriptor offset like a row shift.  An MMA of 128 rows takes the tensor
 // pipe 64 cycles at N = 128, 48 at 64 and still 44 at 32, so a CTA holds as many columns as fit:
 // all nine taps up to N = 56, else the three taps of one kernel row with up to 128 columns
-// (nine taps of 32 columns before: layers 2-5 at batch 64 took 96, 212, 212 and 600 us).
+// (nine taps of 32 columns before: layers 2-5 at batch 64 took 96, ~212, ~212 and 600 us, now
+// 47, 55, 84 and 128).
 // A CTA runs over a strided subset of the pixel tiles and writes its partial sums;
 // k_wgrad_reduce adds them in a fixed order.  Rows beyond the real channel count read whatever
 // lies next in shared memory and are discarded.
@@ -336,6 +408,7 @@ struct WgArgs {
     int planes, rows, N, c_tiles, tmem_cols, n_stage;
     int g_slot, x_slot, g_bytes, x_bytes, stage_bytes;
     int n_split;      // gridDim.x
+    uint32_t tap_at[3][4][9];   // kernel row (0 if all), phase, tap: offset of its input in a stage, 16-byte units
     int Co, Ci;
     float* part;
     unsigned* err;
@@ -359,29 +432,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tc(const __grid_constant_
     __shared__ uint64_t full[kMaxStage], empty[kMaxStage], done;
     __shared__ uint32_t tbase;
     __shared__ int abort_flag, issued, consumed;
-    __shared__ uint32_t tap_at[4][9];   // phase, tap: offset of its input pixels in a stage, 16-byte units
     const WgArgs& a = p.a;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int split = blockIdx.x, kind = blockIdx.y;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int split = blockIdx.x, kind = blockIdx.y * gridDim.z + blockIdx.z;
     const int S = a.n_stage;
-    const int u0 = a.taps == 3 ? kind % 3 : -1;            // the kernel row, -1: all
-    const int tile_kind = a.taps == 3 ? kind / 3 : kind;
-    const int mt = tile_kind / a.c_tiles, nt = tile_kind % a.c_tiles;
+    const int u0 = a.taps == 3 ? (int)blockIdx.z : -1;     // the kernel row, -1: all
+    const int mt = blockIdx.y / a.c_tiles, nt = blockIdx.y % a.c_tiles;
     const int o0 = a.w2 ? nt * a.N : mt * 128, c0 = a.w2 ? mt * 128 : nt * a.N;
-    for (int i = threadIdx.x; i < a.phases * a.taps; i += kThreads) {
-        const int ph = i / a.taps, t = i % a.taps, u = a.taps == 3 ? u0 : t / 3, v = t % 3;
-        int plane, row, col;
-        if (a.up) {
-            plane = 0;
-            row = a.taps == 3 ? 0 : tap_shift(ph >> 1, u) + 1;
-            col = tap_shift(ph & 1, v) + 1;
-        } else {
-            plane = (a.taps == 3 ? 0 : 2 * (u != 1)) + (v != 1);
-            row = a.taps == 3 ? 0 : (u == 0 ? 0 : 1);
-            col = v == 0 ? 0 : 1;
-        }
-        tap_at[ph][t] = (uint32_t)(a.g_bytes + plane * a.x_real * a.x_slot + row * kWgPitch + col * 16) >> 4;
-    }
     const int per_phase = a.tiles_x * a.tiles_y;
 
     if (warp == 0) tmem_alloc(smem_u32(&tbase), a.tmem_cols);
@@ -399,32 +456,29 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tc(const __grid_constant_
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tmem = tbase;
-    const uint32_t sbase = smem_u32(smem);
-    const int my_tiles = split < a.n_tiles ? (a.n_tiles - 1 - split) / a.n_split + 1 : 0;
+    const uint32_t tmem = (uint32_t)uniform((int)tbase);
+    const uint32_t sbase = (uint32_t)uniform((int)smem_u32(smem));
+    const int my_tiles = split < a.n_tiles ? (a.n_tiles - 1 - split) / a.n_split + 1 : 0;   // in each phase
 
     if (warp == 0) {
-        // TMA producer: lane 0 issues, the other lanes wait at the warp barrier
-        if (lane == 0) {
-            int it = 0;
-            for (; it < my_tiles; ++it) {
-                const int tile = split + it * a.n_split;
-                const int nimg = tile / (a.phases * per_phase), rem = tile % (a.phases * per_phase);
-                const int ph = rem / per_phase, tt = rem % per_phase;
-                const int a0 = (tt / a.tiles_x) * a.rows_px, b0 = (tt % a.tiles_x) * 16;
-                const int s = it % S, use = it / S;
-                if (use > 0 && !bar_wait(smem_u32(&empty[s]), (use - 1) & 1, a.spin)) {
+        if (elect_one()) {   // TMA producer
+            const uint32_t bytes = (uint32_t)(2 * (a.g_real * a.g_slot + a.planes * a.x_real * a.rows * kWgPitch));
+            int it = 0, s = 0;
+            uint32_t par = 1;   // a fresh barrier's previous phase counts as complete
+            for (int i = 0; i < a.phases * my_tiles; ++i, ++it) {
+                const int ph = i / my_tiles, tile = split + (i - ph * my_tiles) * a.n_split;
+                const int nimg = tile / per_phase, tt = tile - nimg * per_phase, ty = tt / a.tiles_x;
+                const int a0 = ty * a.rows_px, b0 = (tt - ty * a.tiles_x) * 16;
+                if (!bar_wait(smem_u32(&empty[0]) + 8 * s, par, a.spin)) {
                     atomicOr(a.err, 8u);
                     abort_flag = 1;
                     break;
                 }
                 if (*(volatile int*)&abort_flag) break;
-                const uint32_t bytes = (uint32_t)(2 * (a.g_real * a.g_slot + a.planes * a.x_real * a.rows * kWgPitch));
-                const uint32_t st = sbase + s * a.stage_bytes;
-                const uint32_t fb = smem_u32(&full[s]);
-                bar_expect_tx(fb, bytes);
+                const uint32_t st = sbase + s * a.stage_bytes, fb = smem_u32(&full[0]) + 8 * s;
                 // first input row: all nine taps start one row up, one kernel row at its own
                 const int row0 = u0 < 0 ? a0 - 1 : a0 + (a.up ? tap_shift(ph >> 1, u0) : (u0 == 0 ? -1 : 0));
+                bar_expect_tx(fb, bytes);
                 for (int sp = 0; sp < 2; ++sp) {
                     for (int q = 0; q < a.g_real; ++q) {
                         const int chunk = (o0 >> 3) + q;
@@ -433,63 +487,65 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tc(const __grid_constant_
                     }
                     for (int pl = 0; pl < a.planes; ++pl) {
                         // parity plane (qy, qx) of a stride-2 layer's input: pl = 2 qy + qx, or qx with qy = (u0 != 1)
-                        const int par = u0 < 0 ? pl : 2 * (u0 != 1) + pl;
+                        const int pq = u0 < 0 ? pl : 2 * (u0 != 1) + pl;
                         const uint32_t xb = st + (uint32_t)(a.g_bytes + ((sp * a.planes + pl) * a.x_real) * a.x_slot);
                         for (int q = 0; q < a.x_real; ++q) {
                             const int chunk = (c0 >> 3) + q;
                             tma_load_4d(xb + (uint32_t)(q * a.x_slot), &p.xmap[sp], (b0 - 1) * 8, row0,
-                                        a.up ? chunk : 4 * chunk + par, nimg, fb);
+                                        a.up ? chunk : 4 * chunk + pq, nimg, fb);
                         }
                     }
                 }
+                if (++s == S) s = 0, par ^= 1u;
             }
             issued = it;
         }
         __syncwarp();
     } else if (warp == 1) {
-        // MMA issuer: lane 0 issues, the other lanes wait at the warp barrier
-        if (lane == 0) {
+        if (elect_one()) {
+            // MMA issuer: as in k_conv_tc, every operand is formed from parameters, loop counters and
+            // block indices
             const uint32_t idesc = idesc_bf16(128, a.N, 1, 1);
-            int it = 0;
-            for (; it < my_tiles; ++it) {
-                const int tile = split + it * a.n_split;
-                const int ph = (tile % (a.phases * per_phase)) / per_phase;
-                const int s = it % S, use = it / S;
-                if (!bar_wait(smem_u32(&full[s]), use & 1, a.spin)) {
-                    atomicOr(a.err, 16u);
-                    abort_flag = 1;
-                    break;
-                }
-                fence_after();
-                // operand offsets in the descriptors' 16-byte units, added to the stage's two
-                // descriptors (the issuing thread's time per MMA has to stay below the pipe's):
-                // the layers' gradients at batch 64 1389 -> 1284 us in all
-                const uint32_t st = sbase + s * a.stage_bytes;
-                const uint64_t gd0 = sdesc(st, 128u, (uint32_t)a.g_slot);
-                const uint64_t xd0 = sdesc(st, 128u, (uint32_t)a.x_slot);
-                const uint32_t xlo = (uint32_t)(a.planes * a.x_real * a.x_slot) >> 4;  // hi -> lo half
-                const uint32_t glo = (uint32_t)(a.g_real * a.g_slot) >> 4;
-                for (int tap = 0; tap < a.taps; ++tap) {
-                    const uint32_t d = tmem + (uint32_t)(tap * a.N);
-                    uint64_t gh = gd0, xh = xd0 + tap_at[ph][tap];
-                    uint32_t acc = it > 0;
-#pragma unroll 4
-                    for (int k = 0; k < a.rows_px; ++k, gh += 16, xh += kWgPitch / 16) {   // a row of 16 dy pixels is 256 bytes
-                        const uint64_t gl = gh + glo, xl = xh + xlo;
-                        if (a.w2) {
-                            mma_bf16(d, xh, gh, idesc, acc);
-                            mma_bf16(d, xl, gh, idesc, 1u);
-                            mma_bf16(d, xh, gl, idesc, 1u);
-                        } else {
-                            mma_bf16(d, gh, xh, idesc, acc);
-                            mma_bf16(d, gh, xl, idesc, 1u);
-                            mma_bf16(d, gl, xh, idesc, 1u);
-                        }
-                        acc = 1u;
+            const uint32_t xlo = (uint32_t)(a.planes * a.x_real * a.x_slot) >> 4;  // hi -> lo half
+            const uint32_t glo = (uint32_t)(a.g_real * a.g_slot) >> 4;
+            int it = 0, s = 0;
+            uint32_t par = 0, acc0 = 0u;
+            bool gone = false;
+            for (int ph = 0; ph < a.phases && !gone; ++ph)
+                for (int i = 0; i < my_tiles; ++i, ++it) {
+                    if (!bar_wait(smem_u32(&full[0]) + 8 * s, par, a.spin)) {
+                        atomicOr(a.err, 16u);
+                        abort_flag = 1;
+                        gone = true;
+                        break;
                     }
+                    fence_after();
+                    const uint32_t st = sbase + s * a.stage_bytes;
+                    const uint64_t gd0 = sdesc(st, 128u, (uint32_t)a.g_slot);
+                    const uint64_t xd0 = sdesc(st, 128u, (uint32_t)a.x_slot);
+                    for (int tap = 0; tap < a.taps; ++tap) {
+                        const uint32_t d = tmem + (uint32_t)(tap * a.N);
+                        uint64_t gh = gd0, xh = xd0 + a.tap_at[blockIdx.z][ph][tap];
+                        uint32_t acc = acc0;
+#pragma unroll 4
+                        for (int k = 0; k < a.rows_px; ++k, gh += 16, xh += kWgPitch / 16) {   // a row of 16 dy pixels is 256 bytes
+                            const uint64_t gl = gh + glo, xl = xh + xlo;
+                            if (a.w2) {   // hi.hi, hi.lo, lo.hi
+                                mma_bf16(d, xh, gh, idesc, acc);
+                                mma_bf16(d, xl, gh, idesc, 1u);
+                                mma_bf16(d, xh, gl, idesc, 1u);
+                            } else {
+                                mma_bf16(d, gh, xh, idesc, acc);
+                                mma_bf16(d, gh, xl, idesc, 1u);
+                                mma_bf16(d, gl, xh, idesc, 1u);
+                            }
+                            acc = 1u;
+                        }
+                    }
+                    acc0 = 1u;
+                    mma_commit(smem_u32(&empty[0]) + 8 * s);
+                    if (++s == S) s = 0, par ^= 1u;
                 }
-                mma_commit(smem_u32(&empty[s]));
-            }
             consumed = it;
             mma_commit(smem_u32(&done));
         }
@@ -673,7 +729,6 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 EncodeTiledFn g_encode = nullptr;
 bool g_ready = false;
 int g_conv_dyn = 0, g_wg_dyn = 0;   // dynamic shared memory the two kernels may request
-int g_conv_half = 0;                // ... and k_conv_tc with two CTAs on an SM
 
 // map of one half (hi or lo) of a chunk-major tensor; box = `px` pixels x 8 channels x `rows`
 // rows of one chunk (one parity plane of a parity-split tensor: chunk coordinate 4 q + plane)
@@ -715,11 +770,10 @@ void sort_groups(ConvArgs& a, const Group* g, int ng, int phases) {
 
 // stages and tile sizes for a given N; returns false when not even one stage fits
 bool fit_stages(ConvArgs& a) {
-    a.a_slot = a.rows * 256;
+    a.a_slot = (a.rows * a.px * 16 + 127) / 128 * 128;   // a TMA load's destination: 128-byte aligned
     a.a_bytes = a.split * a.n_copy * 2 * a.a_slot;
     a.stage_bytes = a.a_bytes + 2 * 9 * a.N * 16;
-    const int budget = g_conv_dyn - 1024;
-    a.n_stage = std::min(kMaxStage, std::min(a.ksteps, budget / a.stage_bytes));
+    a.n_stage = std::min(kMaxStage, (g_conv_dyn - 1024) / a.stage_bytes);
     return a.n_stage >= 1;
 }
 
@@ -731,7 +785,7 @@ cudaError_t finish_plan(ConvPlan& pl, int n_img, int num_sms, int phases, int Nt
         if (Ntot % N) continue;
         a.N = N;
         if (!fit_stages(a)) continue;
-        if (a.n_stage >= std::min(2, a.ksteps)) {
+        if (a.n_stage >= 2) {
             best = N;
             break;
         }
@@ -740,31 +794,28 @@ cudaError_t finish_plan(ConvPlan& pl, int n_img, int num_sms, int phases, int Nt
     if (!best) return cudaErrorInvalidConfiguration;
     a.N = best;
     fit_stages(a);
-    // phases per CTA: all of them if TMEM allows and the grid still covers the SMs
+    // phases per tile: all of them if two sets of accumulators fit in TMEM and the tiles still
+    // cover the SMs
     const int tiles = a.tiles_x * a.tiles_y * n_img * (Ntot / a.N);
     a.P = phases;
-    while (a.P > 1 && (a.P * a.N > 512 || tiles * (phases / a.P) < num_sms)) a.P >>= 1;
+    while (a.P > 1 && (2 * a.P * a.N > 512 || tiles * (phases / a.P) < num_sms)) a.P >>= 1;
+    a.n_acc = 2 * a.P * a.N <= 512 ? 2 : 1;
     if (a.P * a.N > 512) return cudaErrorInvalidConfiguration;
-    a.tmem_cols = pow2_cols(a.P * a.N);
-    // Two CTAs per SM where their accumulators fit in TMEM together (and a stage of each in
-    // shared memory): one CTA's set-up and epilogue then overlap the other's MMAs.
-    if (a.tmem_cols <= 256) {
-        const int half = (g_conv_half - 1024) / a.stage_bytes;
-        if (half >= 1) a.n_stage = std::min(a.n_stage, half);
+    a.tmem_cols = pow2_cols(a.n_acc * a.P * a.N);
+    for (int i = 0; i < a.gstart[phases] * a.split; ++i) {
+        const Group gr = a.group[i / a.split];
+        const int sp = i % a.split;
+        const bool first = sp == 0 && i / a.split == a.gstart[gr.phase];
+        pl.prm.mma[i] = make_uint4((unsigned)((sp * a.n_copy + gr.copy) * 2 * a.a_slot + (gr.row * a.px + gr.col) * 16) >> 4,
+                                   (unsigned)(gr.tap * 2 * a.N * 16) >> 4, (unsigned)(gr.phase % a.P * a.N), first ? 0u : 1u);
     }
-    for (int pg = 0; pg < 4; ++pg) {
-        unsigned m = 0;
-        if (pg < phases / a.P)
-            for (int g = a.gstart[pg * a.P]; g < a.gstart[pg * a.P + a.P]; ++g) m |= 1u << a.group[g].copy;
-        a.cmask[pg] = m;
-    }
-    pl.grid = dim3(a.tiles_x * a.tiles_y * n_img, phases / a.P, Ntot / a.N);
-    int smem = a.n_stage * a.stage_bytes + 1024;
-    // more than 256 TMEM columns: keep one CTA per SM so the allocation never waits
-    if (a.tmem_cols > 256) smem = std::max(smem, kOneCtaPerSm);
-    if (smem > g_conv_dyn) return cudaErrorInvalidConfiguration;
-    pl.smem = smem;
-    return cudaSuccess;
+    a.n_img = n_img;
+    a.pgroups = phases / a.P;
+    a.n_zt = Ntot / a.N;
+    pl.grid = dim3(std::min(std::max(1, num_sms / a.pgroups), tiles), a.pgroups);
+    // one CTA per SM, so that its TMEM allocation never waits
+    pl.smem = std::max(a.n_stage * a.stage_bytes + 1024, kOneCtaPerSm);
+    return pl.smem > g_conv_dyn ? cudaErrorInvalidConfiguration : cudaSuccess;
 }
 
 }  // namespace
@@ -782,10 +833,6 @@ cudaError_t tc_prepare() {
     cudaFuncAttributes fa;
     if ((e = cudaFuncGetAttributes(&fa, k_conv_tc)) != cudaSuccess) return e;
     g_conv_dyn = std::min(kSmemLimit, optin - (int)fa.sharedSizeBytes);
-    int per_sm = 0, reserved = 0;
-    if ((e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev)) != cudaSuccess) return e;
-    g_conv_half = per_sm / 2 - reserved - (int)fa.sharedSizeBytes;
     if ((e = cudaFuncGetAttributes(&fa, k_wgrad_tc)) != cudaSuccess) return e;
     g_wg_dyn = std::min(kSmemLimit, optin - (int)fa.sharedSizeBytes);
     if ((e = cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, g_conv_dyn)) != cudaSuccess) return e;
@@ -810,33 +857,32 @@ cudaError_t tc_conv_forward(const TcLayer& L, const Act2& x, const __nv_bfloat16
         // the input is read by parity planes: it must be stored split by parity
         if (!x.par) return cudaErrorInvalidValue;
         phases = 1;
-        a.tiles_y = Ho / 8;
-        a.tiles_x = Ho / 16;
-        a.rows = 9;
-        a.n_copy = 6;
-        const int qx[3] = {0, 1, 1}, dx[3] = {0, -1, 0};
-        for (int qy = 0; qy < 2; ++qy)
-            for (int var = 0; var < 3; ++var) a.copy[qy * 3 + var] = Copy{-1, (int8_t)dx[var], (int8_t)(2 * qy + qx[var])};
+        a.tiles_y = Ho / 16;
+        a.tiles_x = Ho / 8;
+        a.rows = 17;
+        a.px = 9;
+        a.n_copy = 4;
+        for (int pl4 = 0; pl4 < 4; ++pl4) a.copy[pl4] = Copy{-1, -1, (int8_t)pl4};
         for (int u = 0; u < 3; ++u)
-            for (int v = 0; v < 3; ++v) {
-                const int qy = u == 1 ? 0 : 1, dy = u == 0 ? -1 : 0, var = v == 1 ? 0 : (v == 0 ? 1 : 2);
-                g[ng++] = Group{0, (uint8_t)(qy * 3 + var), (uint8_t)(dy + 1), (uint8_t)(3 * u + v)};
-            }
+            for (int v = 0; v < 3; ++v)
+                g[ng++] = Group{0, (uint8_t)(2 * (u != 1) + (v != 1)), (uint8_t)(u == 0 ? 0 : 1), (uint8_t)(v == 0 ? 0 : 1),
+                                (uint8_t)(3 * u + v)};
         a.osy = a.osx = 1;
     } else {
         phases = 4;
-        a.tiles_y = L.Hin / 8;
-        a.tiles_x = L.Hin / 16;
+        a.tiles_y = L.Hin / 16;
+        a.tiles_x = L.Hin / 8;
         if (x.par) return cudaErrorInvalidValue;
-        a.rows = 10;
-        a.n_copy = 3;
-        for (int j = 0; j < 3; ++j) a.copy[j] = Copy{-1, (int8_t)(j - 1), -1};
+        a.rows = 18;
+        a.px = 10;
+        a.n_copy = 1;
+        a.copy[0] = Copy{-1, -1, -1};
         for (int py = 0; py < 2; ++py)
             for (int px = 0; px < 2; ++px)
                 for (int u = 0; u < 3; ++u)
                     for (int v = 0; v < 3; ++v)
-                        g[ng++] = Group{(uint8_t)(2 * py + px), (uint8_t)(half_shift(px, v) + 1),
-                                        (uint8_t)(half_shift(py, u) + 1), (uint8_t)(3 * u + v)};
+                        g[ng++] = Group{(uint8_t)(2 * py + px), 0, (uint8_t)(half_shift(py, u) + 1),
+                                        (uint8_t)(half_shift(px, v) + 1), (uint8_t)(3 * u + v)};
         a.osy = a.osx = 2;
         for (int ph = 0; ph < 4; ++ph) {
             a.opy[ph] = (int8_t)(ph >> 1);
@@ -847,7 +893,7 @@ cudaError_t tc_conv_forward(const TcLayer& L, const Act2& x, const __nv_bfloat16
     const bool last = y == nullptr;
     const int Ntot = (L.Co + 15) / 16 * 16;
     if ((e = finish_plan(pl, x.N, num_sms, phases, Ntot)) != cudaSuccess) return e;
-    if (!enc_act(&pl.prm.amap[0], x.hi, x, x.par != 0, a.rows) || !enc_act(&pl.prm.amap[1], x.lo, x, x.par != 0, a.rows))
+    if (!enc_act(&pl.prm.amap[0], x.hi, x, x.par != 0, a.rows, a.px) || !enc_act(&pl.prm.amap[1], x.lo, x, x.par != 0, a.rows, a.px))
         return cudaErrorInvalidValue;
     a.wts = wf;
     a.wK8 = L.Ci_pad / 8;
@@ -866,7 +912,7 @@ cudaError_t tc_conv_forward(const TcLayer& L, const Act2& x, const __nv_bfloat16
     a.relu = L.relu;
     a.err = err;
     a.spin = spin;
-    k_conv_tc<<<pl.grid, kThreads, pl.smem, st>>>(pl.prm);
+    k_conv_tc<<<pl.grid, kConvThreads, pl.smem, st>>>(pl.prm);
     return cudaGetLastError();
 }
 
@@ -893,18 +939,19 @@ cudaError_t tc_conv_backward_data(const TcLayer& L, const Act2& dy, const __nv_b
         // dx on the input grid in four parity phases; dy rows a'+e, columns b'+f
         phases = 4;
         const int Sd = L.Hin / 2;
-        a.tiles_y = Sd / 8;
-        a.tiles_x = Sd / 16;
-        a.rows = 9;
-        a.n_copy = 2;
-        for (int j = 0; j < 2; ++j) a.copy[j] = Copy{0, (int8_t)j, -1};
+        a.tiles_y = Sd / 16;
+        a.tiles_x = Sd / 8;
+        a.rows = 17;
+        a.px = 9;
+        a.n_copy = 1;
+        a.copy[0] = Copy{0, 0, -1};
         for (int qy = 0; qy < 2; ++qy)
             for (int qx = 0; qx < 2; ++qx)
                 for (int u = 0; u < 3; ++u)
                     for (int v = 0; v < 3; ++v) {
                         if ((qy == 0) != (u == 1) || (qx == 0) != (v == 1)) continue;
                         const int ey = (qy == 1 && u == 0) ? 1 : 0, ex = (qx == 1 && v == 0) ? 1 : 0;
-                        g[ng++] = Group{(uint8_t)(2 * qy + qx), (uint8_t)ex, (uint8_t)ey, (uint8_t)(3 * u + v)};
+                        g[ng++] = Group{(uint8_t)(2 * qy + qx), 0, (uint8_t)ey, (uint8_t)ex, (uint8_t)(3 * u + v)};
                     }
         a.osy = a.osx = 2;
         for (int ph = 0; ph < 4; ++ph) {
@@ -916,20 +963,22 @@ cudaError_t tc_conv_backward_data(const TcLayer& L, const Act2& dy, const __nv_b
         // stride-1 correlation of dy with the transposed weights, then 2 x 2 sums
         phases = 1;
         const int Sd = L.Hout();
-        a.tiles_y = Sd / 8;
-        a.tiles_x = Sd / 16;
-        a.rows = 10;
-        a.n_copy = 3;
-        for (int j = 0; j < 3; ++j) a.copy[j] = Copy{-1, (int8_t)(j - 1), -1};
+        a.tiles_y = Sd / 16;
+        a.tiles_x = Sd / 8;
+        a.rows = 18;
+        a.px = 10;
+        a.n_copy = 1;
+        a.copy[0] = Copy{-1, -1, -1};
         for (int u = 0; u < 3; ++u)
-            for (int v = 0; v < 3; ++v) g[ng++] = Group{0, (uint8_t)(2 - v), (uint8_t)(2 - u), (uint8_t)(3 * u + v)};
+            for (int v = 0; v < 3; ++v)
+                g[ng++] = Group{0, 0, (uint8_t)(2 - u), (uint8_t)(2 - v), (uint8_t)(3 * u + v)};
         a.osy = a.osx = 1;
         a.mode = EPI_POOL;
     }
     sort_groups(a, g, ng, phases);
     if (dy.par) return cudaErrorInvalidValue;   // both forms read dy by plain rows
     if ((e = finish_plan(pl, dy.N, num_sms, phases, L.Ci)) != cudaSuccess) return e;
-    if (!enc_act(&pl.prm.amap[0], dy.hi, dy, false, a.rows) || !enc_act(&pl.prm.amap[1], dy.lo, dy, false, a.rows))
+    if (!enc_act(&pl.prm.amap[0], dy.hi, dy, false, a.rows, a.px) || !enc_act(&pl.prm.amap[1], dy.lo, dy, false, a.rows, a.px))
         return cudaErrorInvalidValue;
     a.wts = wb;
     a.wK8 = L.Co_pad / 8;
@@ -948,8 +997,8 @@ cudaError_t tc_conv_backward_data(const TcLayer& L, const Act2& dy, const __nv_b
     a.db_part = db_part;
     a.err = err;
     a.spin = spin;
-    *n_part = (int)(pl.grid.x * pl.grid.y);
-    k_conv_tc<<<pl.grid, kThreads, pl.smem, st>>>(pl.prm);
+    *n_part = a.tiles_x * a.tiles_y * a.n_img * a.pgroups;
+    k_conv_tc<<<pl.grid, kConvThreads, pl.smem, st>>>(pl.prm);
     return cudaGetLastError();
 }
 
@@ -1001,7 +1050,7 @@ cudaError_t plan_wgrad(WgPlan& pl, const TcLayer& L, const Act2* x, const Act2* 
     if (a.n_stage < 1) return cudaErrorInvalidConfiguration;
     a.tiles_y = S / a.rows_px;
     a.tiles_x = S / 16;
-    a.n_tiles = n_img * a.phases * a.tiles_x * a.tiles_y;
+    a.n_tiles = n_img * a.tiles_x * a.tiles_y;   // of one phase
     a.n_split = std::max(1, std::min(a.n_tiles, num_sms / kinds));
     if (x && dy) {
         // up layers read dy by parity planes (its parity copy), stride-2 layers by plain rows;
@@ -1014,7 +1063,24 @@ cudaError_t plan_wgrad(WgPlan& pl, const TcLayer& L, const Act2* x, const Act2* 
             !enc_act(&pl.prm.xmap[1], x->lo, *x, x->par != 0, a.rows, kWgPx))
             return cudaErrorInvalidValue;
     }
-    pl.grid = dim3(a.n_split, kinds, 1);
+    const int rows_u = 9 / a.taps;   // kernel rows handled apart
+    for (int ur = 0; ur < rows_u; ++ur)
+        for (int ph = 0; ph < a.phases; ++ph)
+            for (int t = 0; t < a.taps; ++t) {
+                const int u = rows_u == 3 ? ur : t / 3, v = t % 3;
+                int plane, row, col;
+                if (L.up) {
+                    plane = 0;
+                    row = rows_u == 3 ? 0 : half_shift(ph >> 1, u) + 1;
+                    col = half_shift(ph & 1, v) + 1;
+                } else {
+                    plane = (rows_u == 3 ? 0 : 2 * (u != 1)) + (v != 1);
+                    row = rows_u == 3 ? 0 : (u == 0 ? 0 : 1);
+                    col = v == 0 ? 0 : 1;
+                }
+                a.tap_at[ur][ph][t] = (uint32_t)(a.g_bytes + plane * a.x_real * a.x_slot + row * kWgPitch + col * 16) >> 4;
+            }
+    pl.grid = dim3(a.n_split, kinds / rows_u, rows_u);
     pl.smem = a.n_stage * a.stage_bytes + 16 * std::max(a.g_slot, a.x_slot) + 1024;
     if (a.tmem_cols > 256) pl.smem = std::max(pl.smem, kOneCtaPerSm);
     if (pl.smem > g_wg_dyn) return cudaErrorInvalidConfiguration;
@@ -1027,7 +1093,7 @@ size_t tc_wgrad_workspace(const TcLayer& L, int N, int num_sms) {
     if (tc_prepare() != cudaSuccess) return 0;
     static WgPlan pl;
     if (plan_wgrad(pl, L, nullptr, nullptr, N, num_sms) != cudaSuccess) return 0;
-    return (size_t)pl.grid.x * pl.grid.y * pl.prm.a.taps * 128 * pl.prm.a.N;
+    return (size_t)pl.grid.x * pl.grid.y * pl.grid.z * pl.prm.a.taps * 128 * pl.prm.a.N;
 }
 
 cudaError_t tc_conv_wgrad(const TcLayer& L, const Act2& x, const Act2& dy, float* ws, float* dw, unsigned* err,
@@ -1042,7 +1108,7 @@ cudaError_t tc_conv_wgrad(const TcLayer& L, const Act2& x, const Act2& dy, float
     a.spin = spin;
     k_wgrad_tc<<<pl.grid, kThreads, pl.smem, st>>>(pl.prm);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_wgrad_reduce<<<dim3((a.taps * 128 * a.N + 255) / 256, pl.grid.y), 256, 0, st>>>(ws, L.Co, L.Ci, a.w2, a.taps,
+    k_wgrad_reduce<<<dim3((a.taps * 128 * a.N + 255) / 256, pl.grid.y * pl.grid.z), 256, 0, st>>>(ws, L.Co, L.Ci, a.w2, a.taps,
                                                                                     a.c_tiles, a.N, a.n_split, dw);
     return cudaGetLastError();
 }

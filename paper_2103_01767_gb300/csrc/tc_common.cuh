@@ -27,6 +27,9 @@ __device__ __forceinline__ void bar_fence_init() { asm volatile("fence.mbarrier_
 __device__ __forceinline__ void bar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
+__device__ __forceinline__ void bar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
 // true once the phase with the given parity has completed; false after `limit` polls
 __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, uint32_t limit) {
     uint32_t done = 0;
@@ -74,6 +77,19 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n, int a_mn, int b_
            ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
+// The tensor-core and TMA instructions take their operands from uniform registers.  A warp
+// that runs its role as a whole, with operands the compiler can prove uniform (parameters,
+// uniform loop counters, values passed through `uniform`), computes them there; one elected
+// lane issues.  In a branch taken by one lane every operand of every instruction is moved
+// over from vector registers: 109 cycles per MMA of N = 64 instead of 49, 124 instead of 64
+// at N = 128.
+__device__ __forceinline__ uint32_t elect_one() {   // 1 in one lane of the (converged) warp, always the same
+    uint32_t e = 0;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e;
+}
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+
 __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(
@@ -98,15 +114,24 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t base, uint32_t cols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols) : "memory");
 }
 // whole warp: 16 consecutive FP32 columns of the warp's 32 lanes (lane i of the warp reads
-// TMEM lane 32 (warp % 4) + i)
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
+// TMEM lane 32 (warp % 4) + i); the registers are valid after tmem_ld_wait(), which takes
+// them so that no use of theirs can move above it
+__device__ __forceinline__ void tmem_ld16_start(uint32_t taddr, float* v) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
         : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
           "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
         : "r"(taddr)
         : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait16(float* v) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]), "+f"(v[8]),
+                   "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15])::"memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
+    tmem_ld16_start(taddr, v);
+    tmem_ld_wait16(v);
 }
 
 // x = hi + lo with hi = bf16(x), lo = bf16(x - hi): |x - hi - lo| <= 2^-18 |x|
@@ -140,12 +165,11 @@ __device__ __forceinline__ void load_pair8(const __nv_bfloat16* hi, const __nv_b
     for (int j = 0; j < 8; ++j) v[j] = __bfloat162float(h[j]) + __bfloat162float(l[j]);
 }
 
-// m[j] = (hi + lo > 0) of 8 channels
-__device__ __forceinline__ void load_mask8(const __nv_bfloat16* hi, const __nv_bfloat16* lo, size_t o, bool* m) {
-    float v[8];
-    load_pair8(hi, lo, o, v);
+// m[j] = (hi + lo > 0) of 8 channels, given as the chunk's 16 bytes of each half
+__device__ __forceinline__ void mask8(uint4 hi, uint4 lo, bool* m) {
+    const __nv_bfloat16 *h = reinterpret_cast<const __nv_bfloat16*>(&hi), *l = reinterpret_cast<const __nv_bfloat16*>(&lo);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) m[j] = v[j] > 0.0f;
+    for (int j = 0; j < 8; ++j) m[j] = __bfloat162float(h[j]) + __bfloat162float(l[j]) > 0.0f;
 }
 
 }  // namespace tc
