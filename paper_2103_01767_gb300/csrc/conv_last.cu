@@ -13,6 +13,8 @@
 // Activations are the (hi, lo) pairs of the other layers, added in FP32.
 #include "conv_tc.h"
 
+#include <algorithm>
+
 #include "tc_common.cuh"
 
 namespace ptylm {
@@ -43,57 +45,77 @@ __device__ void build_weff(const __nv_bfloat16* __restrict__ wf, int Co, int Ci,
     }
 }
 
-// y32[n][o][2a + py][2b + px] = bias[o] + sum Weff x, one thread per input pixel (n, a, b)
-__global__ void __launch_bounds__(kThreads) k_last_forward(const __nv_bfloat16* __restrict__ xhi,
-                                                          const __nv_bfloat16* __restrict__ xlo, int N, int H, int W,
-                                                          int Ci, int Ci_pad, int Co, const __nv_bfloat16* __restrict__ wf,
-                                                          const float* __restrict__ bias, float* __restrict__ y32) {
+// four channels (8 bytes of each half) of one pixel, as FP32
+__device__ __forceinline__ void load_pair4(const __nv_bfloat16* hi, const __nv_bfloat16* lo, size_t o, float* v) {
+    const uint2 h = __ldg(reinterpret_cast<const uint2*>(hi + o)), l = __ldg(reinterpret_cast<const uint2*>(lo + o));
+    const __nv_bfloat16 *hh = reinterpret_cast<const __nv_bfloat16*>(&h), *ll = reinterpret_cast<const __nv_bfloat16*>(&l);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = __bfloat162float(hh[j]) + __bfloat162float(ll[j]);
+}
+
+// y32[n][o][2a + py][2b + px] = bias[o] + sum Weff x.  One thread takes the input pixels (a, b)
+// and (a, b + 1), b even: the pair shares the weights' shared-memory reads and two thirds of
+// the input's.  The blocks stay on their SM, so that Weff is formed once per block and not
+// once per 256 pixels.  225 maps of 64 x 64 x 64: 307 us with one pixel per thread and a block
+// per 256 pixels.
+__global__ void __launch_bounds__(kThreads, 2) k_last_forward(const __nv_bfloat16* __restrict__ xhi,
+                                                             const __nv_bfloat16* __restrict__ xlo, int N, int H, int W,
+                                                             int Ci, int Ci_pad, int Co, const __nv_bfloat16* __restrict__ wf,
+                                                             const float* __restrict__ bias, float* __restrict__ y32) {
     __shared__ __align__(16) float weff[kMaxCi * 16 * kMaxCo];
     build_weff(wf, Co, Ci, Ci_pad, weff);
     __syncthreads();
-    const long p = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= (long)N * H * W) return;
-    const int n = (int)(p / ((long)H * W)), a = (int)((p / W) % H), b = (int)(p % W);
-    const int C8 = Ci >> 3;
-    float acc[4][kMaxCo];
+    const int C8 = Ci >> 3, W2 = W >> 1, Ho = 2 * H, Wo = 2 * W;
+    const long pairs = (long)N * H * W2;
+    for (long p = (long)blockIdx.x * blockDim.x + threadIdx.x; p < pairs; p += (long)gridDim.x * blockDim.x) {
+        const int n = (int)(p / ((long)H * W2)), a = (int)((p / W2) % H), b = 2 * (int)(p % W2);
+        float acc[2][4][kMaxCo];
 #pragma unroll
-    for (int ph = 0; ph < 4; ++ph)
+        for (int t = 0; t < 2; ++t)
 #pragma unroll
-        for (int o = 0; o < kMaxCo; ++o) acc[ph][o] = o < Co ? bias[o] : 0.0f;
-    for (int q = 0; q < C8; ++q) {
-        float xv[3][3][8];   // source rows a - 1 .. a + 1, columns b - 1 .. b + 1, 8 channels
+            for (int ph = 0; ph < 4; ++ph)
 #pragma unroll
-        for (int dy = 0; dy < 3; ++dy)
+                for (int o = 0; o < kMaxCo; ++o) acc[t][ph][o] = o < Co ? bias[o] : 0.0f;
+#pragma unroll 1
+        for (int q = 0; q < 2 * C8; ++q) {   // four channels at a time
+            float xv[3][4][4];   // source rows a - 1 .. a + 1, columns b - 1 .. b + 2
 #pragma unroll
-            for (int dx = 0; dx < 3; ++dx) {
-                const int y = a + dy - 1, x = b + dx - 1;
-                if (y >= 0 && y < H && x >= 0 && x < W) {
-                    load_pair8(xhi, xlo, chunk_at(0, C8, H, W, n, y, x, q), xv[dy][dx]);
-                } else {
+            for (int dy = 0; dy < 3; ++dy)
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) xv[dy][dx][j] = 0.0f;
+                for (int dx = 0; dx < 4; ++dx) {
+                    const int y = a + dy - 1, x = b + dx - 1;
+                    if (y >= 0 && y < H && x >= 0 && x < W) {
+                        load_pair4(xhi, xlo, chunk_at(0, C8, H, W, n, y, x, q >> 1) + 4 * (q & 1), xv[dy][dx]);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) xv[dy][dx][j] = 0.0f;
+                    }
+                }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float4* wc = reinterpret_cast<const float4*>(weff + (size_t)(4 * q + j) * 16 * kMaxCo);
+#pragma unroll
+                for (int ph = 0; ph < 4; ++ph) {
+                    const int py = ph >> 1, px = ph & 1;
+                    const float4 w01 = wc[2 * ph], w23 = wc[2 * ph + 1];   // (jy, jx) = 00, 01, 10, 11 x (o0, o1)
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        const float s00 = xv[py][px + t][j], s01 = xv[py][px + 1 + t][j];
+                        const float s10 = xv[py + 1][px + t][j], s11 = xv[py + 1][px + 1 + t][j];
+                        acc[t][ph][0] = fmaf(w01.x, s00, fmaf(w01.z, s01, fmaf(w23.x, s10, fmaf(w23.z, s11, acc[t][ph][0]))));
+                        acc[t][ph][1] = fmaf(w01.y, s00, fmaf(w01.w, s01, fmaf(w23.y, s10, fmaf(w23.w, s11, acc[t][ph][1]))));
+                    }
                 }
             }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float4* wc = reinterpret_cast<const float4*>(weff + (size_t)(8 * q + j) * 16 * kMaxCo);
-#pragma unroll
-            for (int ph = 0; ph < 4; ++ph) {
-                const int py = ph >> 1, px = ph & 1;
-                const float4 w01 = wc[2 * ph], w23 = wc[2 * ph + 1];   // (jy, jx) = 00, 01, 10, 11 x (o0, o1)
-                const float s00 = xv[py][px][j], s01 = xv[py][px + 1][j];
-                const float s10 = xv[py + 1][px][j], s11 = xv[py + 1][px + 1][j];
-                acc[ph][0] = fmaf(w01.x, s00, fmaf(w01.z, s01, fmaf(w23.x, s10, fmaf(w23.z, s11, acc[ph][0]))));
-                acc[ph][1] = fmaf(w01.y, s00, fmaf(w01.w, s01, fmaf(w23.y, s10, fmaf(w23.w, s11, acc[ph][1]))));
-            }
         }
-    }
-    const int Ho = 2 * H, Wo = 2 * W;
-    for (int o = 0; o < Co; ++o)
 #pragma unroll
-        for (int py = 0; py < 2; ++py)
-            *reinterpret_cast<float2*>(y32 + (((size_t)n * Co + o) * Ho + 2 * a + py) * Wo + 2 * b) =
-                make_float2(acc[2 * py][o], acc[2 * py + 1][o]);
+        for (int o = 0; o < kMaxCo; ++o)
+#pragma unroll
+            for (int py = 0; py < 2; ++py)
+                if (o < Co)
+                    *reinterpret_cast<float4*>(y32 + (((size_t)n * Co + o) * Ho + 2 * a + py) * Wo + 2 * b) =
+                        make_float4(acc[0][2 * py][o], acc[0][2 * py + 1][o], acc[1][2 * py][o], acc[1][2 * py + 1][o]);
+    }
 }
 
 // dx = (d conv / d x)^T dy, masked by act > 0, written as the pair dx (and its parity copy);
@@ -297,11 +319,12 @@ size_t wgrad_smem(const TcLayer& L, int W) {
 bool tc_last_supported(const TcLayer& L) { return last_layer_shape_ok(L, L.Hin); }
 
 cudaError_t tc_last_forward(const TcLayer& L, const Act2& x, const __nv_bfloat16* wf, const float* bias, float* y32,
-                            cudaStream_t st) {
+                            int num_sms, cudaStream_t st) {
     if (!last_layer_shape_ok(L, x.H) || x.par || x.C != L.Ci || x.H != L.Hin || x.W != L.Hin) return cudaErrorInvalidValue;
-    const long total = (long)x.N * x.H * x.W;
-    if (total == 0) return cudaSuccess;
-    k_last_forward<<<(unsigned)((total + kThreads - 1) / kThreads), kThreads, 0, st>>>(x.hi, x.lo, x.N, x.H, x.W, L.Ci,
+    const long pairs = (long)x.N * x.H * (x.W / 2);
+    if (pairs == 0) return cudaSuccess;
+    const long blocks = std::min<long>(2L * num_sms, (pairs + kThreads - 1) / kThreads);
+    k_last_forward<<<(unsigned)blocks, kThreads, 0, st>>>(x.hi, x.lo, x.N, x.H, x.W, L.Ci,
                                                                                       L.Ci_pad, L.Co, wf, bias, y32);
     return cudaGetLastError();
 }

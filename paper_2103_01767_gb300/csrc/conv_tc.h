@@ -72,7 +72,7 @@ size_t tc_wgrad_workspace(const TcLayer& L, int N, int num_sms);
 // (Co <= 2, Ci a power of two in 8 .. 256, input side a multiple of 16).
 bool tc_last_supported(const TcLayer& L);
 cudaError_t tc_last_forward(const TcLayer& L, const Act2& x, const __nv_bfloat16* wf, const float* bias, float* y32,
-                            cudaStream_t st);
+                            int num_sms, cudaStream_t st);
 cudaError_t tc_last_backward_data(const TcLayer& L, const Act2& dy, const __nv_bfloat16* wf, const Act2& act,
                                   const Act2& dx, float* db_part, int* n_part, cudaStream_t st);
 int tc_last_bias_parts(const TcLayer& L, int N);

@@ -318,10 +318,16 @@ k_jvp(AdjArgs a) {
     TeamCtx<G> c = team_setup<G>(a.tw);
     const float invS = 1.0f / G::S;
     float2* slot = a.scratch + (size_t)(blockIdx.x * G::TEAMS + c.team) * G::M + c.tid;
+    const int stride = gridDim.x * G::TEAMS;
+    const GlobalProbe<G> probe(a.P, c.tid);
     float2 v[G::E];
-    for (int k = blockIdx.x * G::TEAMS + c.team; k < a.K; k += gridDim.x * G::TEAMS) {
+    int k = blockIdx.x * G::TEAMS + c.team;
+    if (k < a.K) {
         const int2 rc = a.pos[k];
-        gather_times_probe<G>(v, a.O, a.P, a.nx, rc.x, rc.y, c.tid);
+        gather_times_probe<G>(v, a.O, probe, a.nx, rc.x, rc.y, c.tid);
+    }
+    for (; k < a.K; k += stride) {
+        const int2 rc = a.pos[k];
         team_fft_fwd<G>(v, c.sm, c.tw, c.tid);
 #pragma unroll
         for (int e = 0; e < G::E; ++e) slot[e * G::T] = v[e];
@@ -337,7 +343,13 @@ k_jvp(AdjArgs a) {
             const float inv_zeta = rsqrtf(ps.x * ps.x + ps.y * ps.y + a.b);
             jv[e] = (ps.x * dps.x + ps.y * dps.y) * inv_zeta;
         }
-        store_natural<G>(jv, reinterpret_cast<float*>(c.sm), a.out_real + (size_t)k * G::M, c.tid);
+        float* out_k = a.out_real + (size_t)k * G::M;
+        if (k + stride < a.K) {   // the next position's gather goes out with these rows
+            const int2 rn = a.pos[k + stride];
+            store_natural_then_gather<G>(jv, reinterpret_cast<float*>(c.sm), out_k, v, a.O, probe, a.nx, rn.x, rn.y, c.tid);
+        } else {
+            store_natural<G>(jv, reinterpret_cast<float*>(c.sm), out_k, c.tid);
+        }
         team_sync<G>();
     }
 }
@@ -396,6 +408,7 @@ k_jvp_phasor(AdjArgs a, const float2* __restrict__ u) {
         const int2 rc = a.pos[k];
         if constexpr (JOINT) gather_joint<G>(v, a.V, a.P, a.VP, a.O, a.nx, rc.x, rc.y, c.tid);
         else gather_times_probe<G>(v, a.V, a.P, a.nx, rc.x, rc.y, c.tid);
+        prefetch_tile_l2(u + (size_t)k * G::M, sizeof(float2) * G::M, c.tid);
         team_fft_fwd<G>(v, c.sm, c.tw, c.tid);
         const float2* uk = u + (size_t)k * G::M + c.tid;
         float jv[G::E];

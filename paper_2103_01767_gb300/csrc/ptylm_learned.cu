@@ -89,6 +89,12 @@ struct ptylm_net {
     float2* tw = nullptr;              // W_m^j
     float2* u = nullptr;               // F(P)/|F(P)| in team order
     float2* P = nullptr;
+    // ptylm_learned_init's sums over one object and its positions, kept from call to call
+    // (one network serves one caller at a time) and grown when a larger object comes
+    float2* num = nullptr;
+    float* den = nullptr;
+    int* idx = nullptr;
+    size_t num_cap = 0, idx_cap = 0;
 };
 
 namespace {
@@ -149,7 +155,8 @@ ptylm_status forward(ptylm_net* n, const float* X, int N) {
     for (int l = 0; l < NL; ++l) {
         const Act2 y = l < NL - 1 ? batch(n->act[l], N) : Act2{};
         if (l == NL - 1 && n->last_cuda_cores)
-            LCUDA_TRY(tc_last_forward(n->L[l], in, n->wf[l], n->params + n->b_off[l], n->out, n->stream));
+            LCUDA_TRY(tc_last_forward(n->L[l], in, n->wf[l], n->params + n->b_off[l], n->out, n->num_sms,
+                                      n->stream));
         else
             LCUDA_TRY(tc_conv_forward(n->L[l], in, n->wf[l], n->params + n->b_off[l], l < NL - 1 ? &y : nullptr, n->out,
                                       n->err, kConvSpin, n->num_sms, n->stream));
@@ -179,6 +186,33 @@ ptylm_status loss_grad(ptylm_net* n, const float* X, const float* T, int N, doub
                                                 n->err, kConvSpin, n->num_sms, n->stream));
             LCUDA_TRY(tc_bias_reduce(n->db_part, parts, n->L[l].Ci, n->db_tmp, n->grads + n->b_off[l - 1], n->stream));
         }
+    }
+    return PTYLM_OK;
+}
+
+// Room for the stitching sums of an object of N pixels and `count` position indices.
+ptylm_status stitch_workspace(ptylm_net* n, size_t N, size_t count) {
+    if (N > n->num_cap) {
+        cudaFree(n->num);   // cudaFree waits for the work that uses it
+        cudaFree(n->den);
+        n->num = nullptr;
+        n->den = nullptr;
+        n->num_cap = 0;
+        if (cudaMalloc(&n->num, sizeof(float2) * N) != cudaSuccess || cudaMalloc(&n->den, sizeof(float) * N) != cudaSuccess) {
+            cudaGetLastError();
+            return lfail(PTYLM_ERR_NOMEM, "stitching workspace of %zu pixels", N);
+        }
+        n->num_cap = N;
+    }
+    if (count > n->idx_cap) {
+        cudaFree(n->idx);
+        n->idx = nullptr;
+        n->idx_cap = 0;
+        if (cudaMalloc(&n->idx, sizeof(int) * count) != cudaSuccess) {
+            cudaGetLastError();
+            return lfail(PTYLM_ERR_NOMEM, "index workspace of %zu positions", count);
+        }
+        n->idx_cap = count;
     }
     return PTYLM_OK;
 }
@@ -490,13 +524,11 @@ ptylm_status ptylm_learned_init(ptylm_ctx* ctx, ptylm_net* n, const ptylm_c64* P
     float eps_abs = 0.0f;
     LSTATUS_TRY(set_probe(n, P, &eps_abs, nullptr));
     const long N = (long)cv.ny * cv.nx;
-    float2* num = nullptr;
-    float* den = nullptr;
-    int* didx = nullptr;
-    cudaError_t e = cudaMalloc(&num, sizeof(float2) * N);
-    if (e == cudaSuccess) e = cudaMalloc(&den, sizeof(float) * N);
-    if (e == cudaSuccess) e = cudaMalloc(&didx, sizeof(int) * std::max(1, count));
-    if (e == cudaSuccess) e = cudaMemcpy(didx, hi.data(), sizeof(int) * std::max(1, count), cudaMemcpyHostToDevice);
+    LSTATUS_TRY(stitch_workspace(n, (size_t)N, (size_t)count));
+    float2* num = n->num;
+    float* den = n->den;
+    int* didx = n->idx;
+    cudaError_t e = count > 0 ? cudaMemcpy(didx, hi.data(), sizeof(int) * count, cudaMemcpyHostToDevice) : cudaSuccess;
     if (e == cudaSuccess) e = cudaMemsetAsync(num, 0, sizeof(float2) * N, n->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(den, 0, sizeof(float) * N, n->stream);
     ptylm_status s = PTYLM_OK;
@@ -510,9 +542,6 @@ ptylm_status ptylm_learned_init(ptylm_ctx* ctx, ptylm_net* n, const ptylm_c64* P
     }
     if (e == cudaSuccess && s == PTYLM_OK) e = stitch_finish(num, den, N, reinterpret_cast<float2*>(O0), n->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(n->stream);
-    cudaFree(num);
-    cudaFree(den);
-    cudaFree(didx);
     if (s != PTYLM_OK) return s;
     LCUDA_TRY(e);
     return check_conv_wait(n);
@@ -522,6 +551,9 @@ ptylm_status ptylm_net_destroy(ptylm_net* n) {
     if (!n) return PTYLM_OK;
     cudaStreamSynchronize(n->stream);
     for (void* p : n->allocs) cudaFree(p);
+    cudaFree(n->num);
+    cudaFree(n->den);
+    cudaFree(n->idx);
     delete n;
     return PTYLM_OK;
 }

@@ -475,6 +475,20 @@ __device__ __forceinline__ void stagger_release(int tid) {
     }
 }
 
+// Natural [S][S] order in the exchange buffer, for per-pixel values that enter or leave the
+// pass-3 layout: float word of frequency (row ky, column kx).  The 32 lanes of a warp that
+// touch one element index hold distinct (k2x, k1y0, low bits of k1x), i.e. rows ky = k1x + E k2x
+// and columns k1y0 + const; pitch and skew send them to 32 distinct banks, and a row of S
+// consecutive columns stays contiguous.  (Rows of S + 1 words, E = 32 rows apart, put four
+// values of k2x on one bank: up to eight-way conflicts.)
+template <class G>
+__host__ __device__ __forceinline__ int nat_word(int ky, int kx) {
+    constexpr int PITCH = G::BY == 16 ? G::S + 16 : G::BY == 4 ? G::S + 4 : G::S + 1;
+    constexpr int SKEW = G::BY == 16 ? 4 : G::BY == 4 ? 2 : 0;
+    static_assert(G::S * PITCH + SKEW * G::BX <= 2 * G::EXW, "fits the exchange buffer");
+    return ky * PITCH + kx + SKEW * (ky >> G::LOG_E);
+}
+
 // ---- whole transforms ------------------------------------------------------------------
 // Forward: v in pass-1 layout (natural spatial data)  ->  v in pass-3 layout (spectrum).
 template <class G>
@@ -482,7 +496,9 @@ __device__ __forceinline__ void team_fft_fwd(float2* v, float2* sm, const float2
     pass1_fwd<G>(v, tw, tid);
     ex1_store_from_p1<G>(sm, v, tid);
     team_sync<G>();
+    stagger_wait<G>(tid);
     ex1_load_to_p2<G>(sm, v, tid);
+    stagger_release<G>(tid);
     pass2_fwd<G>(v, tw, tid);
     if constexpr (G::BY > 1) {
         ex2_store_from_p2<G>(sm, v, tid);  // into the slots this thread has just read
