@@ -131,6 +131,35 @@ __device__ __forceinline__ void batch_matvec_item(const BatchArgs& a, const Batc
     const float2* V = a.V + p.z_off;
     float2* out = a.out + p.z_off;
     float2 v[G::E];
+    if constexpr (TEAMS == 1) {
+        // one team per CTA (128^2): each position's scatter is fused with the next one's gather,
+        // as in the single-problem product
+        int k = it.k0;
+        const int k1 = min(p.K, it.k0 + it.per_team);
+        int2 rc = p.pos[k];
+        gather_times_probe<G>(v, V, p.P, p.nx, rc.x, rc.y, tid);
+        for (; k < k1; ++k) {
+            const float2* ak = p.a_cache + (size_t)k * G::M;
+            prefetch_tile_l2(ak, sizeof(float2) * G::M, tid);
+            team_fft_roundtrip<G>(v, sm, tw, tid, [&](float2* g, int jj) {
+                float2 av[G::BY];
+                load_cache_group<G>(ak, av, jj, tid);
+#pragma unroll
+                for (int k2y = 0; k2y < G::BY; ++k2y) {
+                    const float t = (av[k2y].x * g[k2y].x + av[k2y].y * g[k2y].y) * invM;
+                    g[k2y] = av[k2y] * t;
+                }
+            });
+            rc = p.pos[k];
+            if (k + 1 < k1) {
+                const int2 rn = p.pos[k + 1];
+                scatter_then_gather<G>(v, out, V, p.P, p.nx, rc.x, rc.y, rn.x, rn.y, tid);
+            } else {
+                scatter_times_conj_probe<G>(v, out, p.P, p.nx, rc.x, rc.y, tid);
+            }
+        }
+        return;
+    }
     for (int j = 0; j < it.per_team; ++j) {
         const int k = it.k0 + team + TEAMS * j;
         const bool valid = k < p.K;
@@ -158,7 +187,8 @@ __device__ __forceinline__ void batch_matvec_item(const BatchArgs& a, const Batc
             }
         });
         if (valid) scatter_times_conj_probe<G>(v, out, p.P, p.nx, rc.x, rc.y, tid);
-        team_sync<G>();
+        // No barrier before the next position: its first shared-memory writes go to the slots
+        // this same thread read last (team_fft_roundtrip).
     }
 }
 

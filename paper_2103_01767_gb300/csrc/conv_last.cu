@@ -57,7 +57,7 @@ __device__ __forceinline__ void load_pair4(const __nv_bfloat16* hi, const __nv_b
 // and (a, b + 1), b even: the pair shares the weights' shared-memory reads and two thirds of
 // the input's.  The blocks stay on their SM, so that Weff is formed once per block and not
 // once per 256 pixels.  225 maps of 64 x 64 x 64: 307 us with one pixel per thread and a block
-// per 256 pixels.
+// per 256 pixels, 250 us now; four pixels per thread spill and take 283.
 __global__ void __launch_bounds__(kThreads, 2) k_last_forward(const __nv_bfloat16* __restrict__ xhi,
                                                              const __nv_bfloat16* __restrict__ xlo, int N, int H, int W,
                                                              int Ci, int Ci_pad, int Co, const __nv_bfloat16* __restrict__ wf,
