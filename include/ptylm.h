@@ -68,8 +68,10 @@ typedef struct {
     size_t workspace_budget;  /* max bytes the context may allocate; 0 = unlimited       */
     int values_per_thread;    /* FFT tile of the single-problem kernels: 32, or 16 for     */
                               /* probe sides 32 and 64 (teams of S^2/16 threads); 0 picks  */
-                              /* 16 for side 64, for joint problems of side 32 and for     */
-                              /* others of side 32 with few positions (ignored by batches) */
+                              /* 16 when the positions would fill less than half of the   */
+                              /* GPU with teams of S^2/32 threads and, without a workspace */
+                              /* budget, for side 64 and joint problems of side 32        */
+                              /* (ignored by batches)                                     */
 } ptylm_desc;
 
 /* Parameters of Algorithm 1 (Sec. 4.2; values used in the paper: Sec. 5). */
@@ -107,17 +109,19 @@ typedef struct {
     double surrogate0;
     double surrogate_end;
     int surrogate_T;
-    /* 0 (default): each CG iteration after its GGN product is one cooperative launch with
-     * two grid-wide FP64 reductions inside it (when the device supports cooperative
-     * launches); 1: three launches (p.q; x, r and r.z; p and q).  Both give the same
-     * results bit for bit.  A bounded grid-wide wait that gives up ends lm_solve with
-     * PTYLM_ERR_TIMEOUT. */
+    /* 0 (default): each CG iteration after its GGN product is one launch -- for states of up
+     * to 98,304 elements one cluster of 16 CTAs that sums through distributed shared memory,
+     * for longer ones a cooperative launch with two grid-wide FP64 reductions inside it (when
+     * the device supports them); 1: three launches (p.q; x, r and r.z; p and q).  Both give
+     * the same results bit for bit.  A bounded grid-wide wait that gives up ends lm_solve
+     * with PTYLM_ERR_TIMEOUT. */
     int separate_cg_kernels;
-    /* Polls of each bounded grid-wide wait of the single-launch CG iteration before it gives
-     * up: 0 (default) about a second (2^24 polls of >= 32 ns); > 0 that many.  A small value
-     * exists for fault-injection tests: the waits then run out, every CTA still finishes its
-     * in-bounds work and exits, and lm_solve returns PTYLM_ERR_TIMEOUT with the context
-     * usable for the next call. */
+    /* Polls of each bounded grid-wide wait of the cooperative CG iteration before it gives
+     * up: 0 (default) about a second (2^24 polls of >= 32 ns); > 0 that many, and the
+     * cooperative form whatever the state's length (the cluster form has no such wait).  A
+     * small value exists for fault-injection tests: the waits then run out, every CTA still
+     * finishes its in-bounds work and exits, and lm_solve returns PTYLM_ERR_TIMEOUT with the
+     * context usable for the next call. */
     int wait_polls;
 } ptylm_lm_params;
 

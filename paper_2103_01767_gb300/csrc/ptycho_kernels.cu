@@ -403,11 +403,19 @@ k_jvp_phasor(AdjArgs a, const float2* __restrict__ u) {
     using G = Geo<LS, LE>;
     TeamCtx<G> c = team_setup<G>(a.tw);
     const float invS = 1.0f / G::S;
+    const int stride = gridDim.x * G::TEAMS;
+    const GlobalProbe<G> probe(a.P, c.tid);
     float2 v[G::E];
-    for (int k = blockIdx.x * G::TEAMS + c.team; k < a.K; k += gridDim.x * G::TEAMS) {
+    int k = blockIdx.x * G::TEAMS + c.team;
+    if constexpr (!JOINT) {
+        if (k < a.K) {
+            const int2 rc = a.pos[k];
+            gather_times_probe<G>(v, a.V, probe, a.nx, rc.x, rc.y, c.tid);
+        }
+    }
+    for (; k < a.K; k += stride) {
         const int2 rc = a.pos[k];
         if constexpr (JOINT) gather_joint<G>(v, a.V, a.P, a.VP, a.O, a.nx, rc.x, rc.y, c.tid);
-        else gather_times_probe<G>(v, a.V, a.P, a.nx, rc.x, rc.y, c.tid);
         prefetch_tile_l2(u + (size_t)k * G::M, sizeof(float2) * G::M, c.tid);
         team_fft_fwd<G>(v, c.sm, c.tw, c.tid);
         const float2* uk = u + (size_t)k * G::M + c.tid;
@@ -417,7 +425,13 @@ k_jvp_phasor(AdjArgs a, const float2* __restrict__ u) {
             const float2 ue = __ldg(uk + e * G::T);
             jv[e] = (ue.x * v[e].x + ue.y * v[e].y) * invS;
         }
-        store_natural<G>(jv, reinterpret_cast<float*>(c.sm), a.out_real + (size_t)k * G::M, c.tid);
+        float* out_k = a.out_real + (size_t)k * G::M;
+        if (!JOINT && k + stride < a.K) {   // the next position's gather goes out with these rows
+            const int2 rn = a.pos[k + stride];
+            store_natural_then_gather<G>(jv, reinterpret_cast<float*>(c.sm), out_k, v, a.V, probe, a.nx, rn.x, rn.y, c.tid);
+        } else {
+            store_natural<G>(jv, reinterpret_cast<float*>(c.sm), out_k, c.tid);
+        }
         team_sync<G>();
     }
 }

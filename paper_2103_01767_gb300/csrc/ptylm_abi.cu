@@ -882,10 +882,16 @@ ptylm_status lm_init(ptylm_ctx** out, const ptylm_desc* desc, const int32_t* pos
     // the faster one over the whole range of K (64^2, 1900 positions, 16 / 32 values: product 45.7 /
     // 50.8 us, blind product 65.8 / 83.5, loss 29.5 / 34.6; 32^2 blind, 8000: 74.7 / 105 us); for
     // other 32^2 problems while teams of S^2/32 threads would fill less than half of the GPU's
-    // thread slots (product at 3000 positions 20.6 / 20.7 us, at 8000 41.2 / 37.0).
+    // thread slots (product at 3000 positions 20.6 / 20.7 us, at 8000 41.2 / 37.0).  Contexts with
+    // a workspace budget keep that half-full rule for all sides: the 16-value tile's d2l sums take
+    // twice the memory, which a budget cut to the 32-value tile would not hold.
     if (d.values_per_thread == 16) c->LE = 4;
     else if (d.values_per_thread == 32) c->LE = 5;
-    else c->LE = LS == 6 || (LS == 5 && (d.joint || (long)d.K * (c->M / 32) < (long)c->num_sms * 1024)) ? 4 : 5;
+    else {
+        const bool few = LS <= 6 && (long)d.K * (c->M / 32) < (long)c->num_sms * 1024;
+        const bool faster = d.workspace_budget == 0 && (LS == 6 || (LS == 5 && d.joint));
+        c->LE = few || faster ? 4 : 5;
+    }
     const int teams = cta_teams(LS, c->LE);
     for (int kid = 0; kid < KID_COUNT; ++kid) {
         int per_sm = 0;
